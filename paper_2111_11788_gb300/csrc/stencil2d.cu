@@ -62,6 +62,7 @@ struct Strip {
   int64_t part_idx;
 };
 
+template <int SR = SROWS>
 __device__ __forceinline__ Strip strip_of(const Grid& g) {
   Strip s;
   const int lane = threadIdx.x & 31;
@@ -71,8 +72,8 @@ __device__ __forceinline__ Strip strip_of(const Grid& g) {
   s.N1 = g.n + 1;
   s.c = strip * 30 - 1 + lane;
   s.out = (lane >= 1) && (lane <= 30) && (s.c <= g.n);
-  s.y0 = blockIdx.y * SROWS;
-  s.y1 = min(s.y0 + SROWS, g.n + 1);
+  s.y0 = blockIdx.y * SR;
+  s.y1 = min(s.y0 + SR, g.n + 1);
   s.part_idx = (int64_t)blockIdx.z * g.tiles_s + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * SWARPS + warp;
   return s;
 }
@@ -425,13 +426,34 @@ __device__ __forceinline__ void warp_partial(T v, double* __restrict__ part, int
 }
 
 inline dim3 sgrid(const Grid& g, int64_t B) { return dim3((unsigned)g.sx, (unsigned)g.sy, (unsigned)B); }
+
+// Rows per strip of a launch that leaves no partial sums (A x, the pre-smoother,
+// the post-smoother below the finest level): SROWS, or SROWS_SHORT where the
+// tall strips are fewer warps than the SMs have partitions. A row costs about
+// 0.8 us of dependent FP64 and L2 latency, which a launch of few warps cannot
+// hide (A x of one sample of 45^2: 22.5 us on 32-row strips, 6.1 us on 4-row
+// ones, launch and binding included); every node's value is the same for
+// either height. The height is a template parameter: as a field of the grid it
+// cost 8 to 16 registers a thread and 4% of a batch of 40 samples of 256^2.
+// Launches with partial sums keep SROWS, which fixes the sums' layout.
+constexpr int SROWS_SHORT = 4;
+constexpr int64_t STRIP_WARPS = 4 * 152;
+template <class F>
+void with_strips(const Grid& g, int64_t B, F&& launch) {
+  const int64_t columns = (int64_t)g.sx * SWARPS * B;
+  if (columns * g.sy < STRIP_WARPS)
+    launch(std::integral_constant<int, SROWS_SHORT>{},
+           dim3((unsigned)g.sx, (unsigned)((g.n + SROWS_SHORT) / SROWS_SHORT), (unsigned)B));
+  else
+    launch(std::integral_constant<int, SROWS>{}, sgrid(g, B));
+}
 constexpr int SBLOCK = SWARPS * 32;
 
-template <class T>
+template <class T, int SR>
 __global__ void __launch_bounds__(SBLOCK) k_apply2(Grid g, const T* __restrict__ K,
                                                    const T* __restrict__ X, T* __restrict__ Y,
                                                    Prof prof) {
-  const Strip s = strip_of(g);
+  const Strip s = strip_of<SR>(g);
   const int64_t b = blockIdx.z;
   const T* x = X + b * g.ns;
   T* y = Y + b * g.ns;
@@ -486,7 +508,7 @@ __global__ void __launch_bounds__(SBLOCK) k_pq2(Grid g, const T* __restrict__ K,
 }
 
 // Pre-smoothing from zero and residual: e = W b, r1 = b - A e.
-template <class T, bool C>
+template <class T, bool C, int SR>
 __global__ void __launch_bounds__(SBLOCK) k_mgpre2(Grid g, const T* __restrict__ K, int64_t cs,
                                                    const T* __restrict__ W,
                                                    const T* __restrict__ Bv, T* __restrict__ E,
@@ -494,7 +516,7 @@ __global__ void __launch_bounds__(SBLOCK) k_mgpre2(Grid g, const T* __restrict__
                                                    const int32_t* __restrict__ active, Prof prof) {
   const int64_t b = blockIdx.z;
   if (!active[b]) return;
-  const Strip s = strip_of(g);
+  const Strip s = strip_of<SR>(g);
   const T* w_ = W + b * g.ns;
   const T* bv = Bv + b * g.ns;
   T* e = E + b * g.ns;
@@ -611,7 +633,7 @@ struct Prolong2 {
 };
 
 // out = e' + W (b - A e'), e' = e + P ec; partials of b.out when part != nullptr.
-template <class T, bool C>
+template <class T, bool C, int SR>
 __global__ void __launch_bounds__(SBLOCK) k_mgpost2(Grid g, int64_t nsc, const T* __restrict__ K, int64_t cs,
                                                     const T* __restrict__ W,
                                                     const T* __restrict__ Bv,
@@ -621,7 +643,7 @@ __global__ void __launch_bounds__(SBLOCK) k_mgpost2(Grid g, int64_t nsc, const T
                                                     double* __restrict__ part, Prof prof) {
   const int64_t b = blockIdx.z;
   if (!active[b]) return;
-  const Strip s = strip_of(g);
+  const Strip s = strip_of<SR>(g);
   const int nc = g.n / 2;
   const T* ec = Ec + b * nsc;
   const T* e = E + b * g.ns;
@@ -665,6 +687,7 @@ __global__ void __launch_bounds__(SBLOCK) k_mgpost2(Grid g, int64_t nsc, const T
 // k_mgpost2 for the FP32 inner solve (kappa form), on paired rows with the
 // prolongation streamed as in Prolong2; its own kernel so that it can be
 // held to 56 registers (9 CTAs per SM) without touching the FP64 kernels.
+template <int SR>
 __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, const float* __restrict__ K,
                                                         const float* __restrict__ W,
                                                         const float* __restrict__ Bv,
@@ -674,7 +697,7 @@ __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, con
                                                         double* __restrict__ part, Prof prof) {
   const int64_t b = blockIdx.z;
   if (!active[b]) return;
-  const Strip s = strip_of(g);
+  const Strip s = strip_of<SR>(g);
   const int nc = g.n / 2;
   const float* ec = Ec + b * nsc;
   const float* e = E + b * g.ns;
@@ -689,7 +712,7 @@ __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, con
   // coarse row J. The fetch of a pair loads coarse row J + 1; H(J) is the
   // previous pair's (hprev). Bitwise equal to prolong2_form (the scalings
   // are exact).
-  static_assert(SROWS % 2 == 0, "strips start on even rows");
+  static_assert(SR % 2 == 0, "strips start on even rows");
   const int n = s.n, c = s.c, N1c = nc + 1;
   const bool cin = c >= 1 && c < n;
   const float* __restrict__ ecol = ec + (cin ? (c >> 1) : 0);
@@ -1410,7 +1433,9 @@ cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, con
 
 template <class T>
 cudaError_t apply(cudaStream_t s, const Grid& g, const T* kappa, const T* x, T* y, int64_t B, Prof p) {
-  k_apply2<T><<<sgrid(g, B), SBLOCK, 0, s>>>(g, kappa, x, y, p);
+  with_strips(g, B, [&](auto sr, dim3 grid) {
+    k_apply2<T, decltype(sr)::value><<<grid, SBLOCK, 0, s>>>(g, kappa, x, y, p);
+  });
   return cudaGetLastError();
 }
 
@@ -1473,10 +1498,13 @@ cudaError_t jacobi_z(cudaStream_t s, const Grid& g, const T* winv, const T* r, T
 template <class T>
 cudaError_t mg_pre(cudaStream_t s, const Grid& g, const T* kappa, const T* w, const T* b, T* e,
                    T* r1, const int32_t* active, int64_t B, Prof p, const T* coef) {
-  if (coef)
-    k_mgpre2<T, true><<<sgrid(g, B), SBLOCK, 0, s>>>(g, coef, coef_stride(g), w, b, e, r1, active, p);
-  else
-    k_mgpre2<T, false><<<sgrid(g, B), SBLOCK, 0, s>>>(g, kappa, g.es, w, b, e, r1, active, p);
+  with_strips(g, B, [&](auto sr, dim3 grid) {
+    constexpr int SR = decltype(sr)::value;
+    if (coef)
+      k_mgpre2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coef, coef_stride(g), w, b, e, r1, active, p);
+    else
+      k_mgpre2<T, false, SR><<<grid, SBLOCK, 0, s>>>(g, kappa, g.es, w, b, e, r1, active, p);
+  });
   return cudaGetLastError();
 }
 
@@ -1509,14 +1537,21 @@ template <class T>
 cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* kappa, const T* w,
                     const T* b, const T* e, const T* ec, T* out, const int32_t* active,
                     double* part, int64_t B, Prof p, const T* coef) {
-  if (coef)
-    k_mgpost2<T, true><<<sgrid(g, B), SBLOCK, 0, s>>>(g, coarse.ns, coef, coef_stride(g), w, b, e, ec, out,
-                                                      active, part, p);
-  else if constexpr (sizeof(T) == 4)
-    k_mgpost2f<<<sgrid(g, B), SBLOCK, 0, s>>>(g, coarse.ns, kappa, w, b, e, ec, out, active, part, p);
+  const auto launch = [&](auto sr, dim3 grid) {
+    constexpr int SR = decltype(sr)::value;
+    if (coef)
+      k_mgpost2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, coef, coef_stride(g), w, b, e, ec, out,
+                                                        active, part, p);
+    else if constexpr (sizeof(T) == 4)
+      k_mgpost2f<SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, w, b, e, ec, out, active, part, p);
+    else
+      k_mgpost2<T, false, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, g.es, w, b, e, ec, out,
+                                                         active, part, p);
+  };
+  if (part)
+    launch(std::integral_constant<int, SROWS>{}, sgrid(g, B));
   else
-    k_mgpost2<T, false><<<sgrid(g, B), SBLOCK, 0, s>>>(g, coarse.ns, kappa, g.es, w, b, e, ec, out,
-                                                       active, part, p);
+    with_strips(g, B, launch);
   return cudaGetLastError();
 }
 

@@ -426,3 +426,21 @@ def test_workspace_kept_across_plans_gives_the_same_results(m):
             qf, qc, it = plan.sample_level(2, 0, 5)
         got.append((qf.tolist(), qc.tolist()))
     assert got[1] == got[0] and got[2] == got[0]
+
+
+@pytest.mark.parametrize("n,count", [(3, 4000), (45, 1500), (64, 300), (200, 64)])
+def test_apply_is_the_same_on_every_strip_height(m, n, count):
+    """A x of one sample alone (short strips) and in a batch (tall ones): the same bits."""
+    cfg = m.config(dim=2, n_levels=1, coarse_cells=n)
+    kap = random_element_field(2, n, 1, seed=n, spread=1.0)
+    x = random_node_vectors(2, n, 1, seed=n + 1)
+    ns, es, nn = m.node_stride(2, n), m.elem_stride(2, n), (n + 1) ** 2
+    kd = elem_arrays_to_device(m, 2, n, kap).repeat(count)
+    xd = node_arrays_to_device(m, 2, n, x).repeat(count)
+    one, many = dev(ns), dev(count * ns)
+    with m.Plan(cfg, stream()) as plan:
+        plan.apply(0, kd.data_ptr(), xd.data_ptr(), one.data_ptr(), 1)
+        plan.apply(0, kd.data_ptr(), xd.data_ptr(), many.data_ptr(), count)
+    torch.cuda.synchronize()
+    got = many.reshape(count, ns)[:, :nn]
+    assert torch.equal(got, one[:nn].expand(count, nn))

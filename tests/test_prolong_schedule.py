@@ -135,3 +135,11 @@ def test_textbook_form_is_bilinear_interpolation(n):
             want = f([[j / n, i / n]])[0]
             got = textbook(e.astype(np.float64), ec, i, j)
             assert abs(got - want) <= 1e-15 * (1 + abs(want)), (i, j, got, want)
+
+
+@pytest.mark.parametrize("rows", [4, 8, 16])
+@pytest.mark.parametrize("n", [2, 8, 64])
+def test_the_same_on_shorter_strips(monkeypatch, n, rows):
+    """Launches of few warps use strips of 4, 8 or 16 rows."""
+    monkeypatch.setitem(globals(), "SROWS", rows)
+    test_streamed_prolongation_is_the_textbook_form_bitwise(n)
