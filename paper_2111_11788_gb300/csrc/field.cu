@@ -6,9 +6,10 @@
 // k = (k_z m + k_y) m + k_x. Because Phi is a Kronecker product of per-axis
 // tables F[i, k] = sqrt(theta_k) f_k((i + 1/2) h), the contraction Phi xi is
 // evaluated axis by axis (sum factorisation) in FP64: for each sample a
-// small x-contraction into shared memory, then m FMAs per element and one
-// exp. On GB300 the FP64 exp and FMAs bound the kernel (about 20 GB/s of
-// kappa per TFLOP/s of FP64), not the write of kappa (8 B per element).
+// small x-contraction into shared memory, then per element the last axis's
+// sum (over the even and odd modes of a mirrored pair of elements) and one
+// exp. On GB300 the FP64 exp and FMAs bound the kernel, not the write of
+// kappa (8 B per element).
 #include <algorithm>
 #include <cmath>
 
@@ -19,31 +20,42 @@ namespace {
 
 // exp in FP64 by the table-driven reduction of P. T. P. Tang ("Table-driven
 // implementation of the exponential function in IEEE floating-point
-// arithmetic", ACM TOMS 15(2), 1989), written from the mathematics:
-//   x = (64 k + j) ln2 / 64 + r,  |r| <= ln2 / 128,  0 <= j < 64,
-//   exp(x) = 2^k 2^(j/64) exp(r),  exp(r) = 1 + p(r),
-//   p(r) = r + r^2 (1/2 + r (1/6 + r (1/24 + r / 120)))
-// (the next Taylor term, r^6 / 720, is below 4e-17). ln2 / 64 is split as
-// L1 + L2 with L1 carrying 32 significant bits, so N L1 is exact for the
-// |N| < 2^21 of |x| < 2^14; 2^(j/64) comes from a table of 64 doubles made on
-// the host. About 1 ulp; |x| < 700 (the log-field of the KLE stays far inside).
-__constant__ double c_exp2_tab[64];
+// arithmetic", ACM TOMS 15(2), 1989), written from the mathematics, for a
+// log-field x that is formed as t = x 64 / ln 2 (the factor goes into the small
+// contracted table, not into a multiply per element):
+//   t = N + f, N = 64 k + j, |f| <= 1/2, 0 <= j < 64,
+//   exp(x) = 2^(t/64) = 2^k 2^(j/64) (1 + p), r = f ln2 / 64,
+//   p = r + r^2 / 2 + r^3 / 6 + r^4 / 24 + r^5 / 120
+// (the next Taylor term, r^6 / 720, is below 4e-17), evaluated in f with the
+// powers of ln2 / 64 in its coefficients. N comes from adding 1.5 2^52 (the
+// low word of the sum holds N, taking it off again gives N, and t - N is
+// exact), 2^(j/64) from a table made on the host, and 2^k is added to the
+// exponent field: 9 FP64 operations per element; reducing x itself with ln2 /
+// 64 in two parts, with conversions through the FP64 pipe and a multiply by
+// 2^k, took 13. About 1 ulp beside the rounding of t. Outside the normal
+// range of the result, and for NaN, the library's exp.
+constexpr int EXP_TAB = 64;
+__device__ double g_exp2_tab[EXP_TAB];
 constexpr double kInvLn2x64 = 92.332482616893658071;   // 64 / ln 2
 // ln 2 / 64 = 0.0108304246962491454596... as L1 (32 significant bits) + L2
 constexpr double kLn2d64Hi = 0x1.62e42fee00000p-7;     // 0.01083042469326755963265895843505859375
 constexpr double kLn2d64Lo = 2.9815858269852934627254151261796896e-12;
+constexpr double kR = kLn2d64Hi + kLn2d64Lo;
+constexpr double kRound = 6755399441055744.0;          // 1.5 2^52
+constexpr int kBig = 0x40ef0000;                       // high word of |t| = 64 * 992 (|x| = 687.6)
 
-__device__ __forceinline__ double kle_exp(double x) {
-  const double t = x * kInvLn2x64;
-  const double nf = rint(t);
-  const int N = (int)nf;
-  const double r = fma(-nf, kLn2d64Lo, fma(-nf, kLn2d64Hi, x));
-  const int j = N & 63;
-  const int k = (N - j) >> 6;
-  const double q = fma(r, fma(r, fma(r, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5);
-  const double p = fma(r * r, q, r);
-  const double T = c_exp2_tab[j];
-  return fma(T, p, T) * __longlong_as_double((long long)(k + 1023) << 52);
+__device__ __forceinline__ double kle_exp(double t, const double* tab) {
+  if ((__double2hiint(t) & 0x7fffffff) >= kBig) return exp(t * kR);
+  const double y = t + kRound;
+  const int N = __double2loint(y);
+  const double f = t - (y - kRound);
+  double q = fma(f, kR * kR * kR * kR * kR / 120.0, kR * kR * kR * kR / 24.0);
+  q = fma(f, q, kR * kR * kR / 6.0);
+  q = fma(f, q, kR * kR / 2.0);
+  q = fma(f, q, kR);
+  const double T = tab[N & (EXP_TAB - 1)];
+  const double v = fma(T, f * q, T);
+  return __hiloint2double(__double2hiint(v) + ((N >> 6) << 20), __double2loint(v));
 }
 
 // F[i * m + k] = sqrt(theta_k) f_k(x_i), x_i = (i + 1/2) / n, centred t = x - 1/2:
@@ -67,10 +79,13 @@ __global__ void k_kle_table(int n, int m, const double* __restrict__ omega,
   table[idx] = sqrt(theta[k]) * f;
 }
 
-// Element rows per thread in 2D: a CTA covers 32 columns x 8 * KAP_ROWS rows,
-// so the x-contraction of its columns (m^2 FMAs per column) is shared by 64
-// rows of elements (m FMAs and one exp each).
-constexpr int KAP_ROWS = 8;
+// Row pairs per thread in 2D. The eigenfunctions are even or odd about the
+// centre, so element rows iy and n - 1 - iy share the sums over the even and
+// over the odd modes, E and O: their fields are E + O and E - O, m / 2 + 1
+// FP64 operations per element instead of m. A CTA covers 32 columns x 8 *
+// KAP_ROWS row pairs, so the x-contraction of its columns (m^2 FMAs per
+// column) is shared by 64 rows.
+constexpr int KAP_ROWS = 4;
 
 // The sample's KLE coefficients in the full tensor layout (m^dim entries) in
 // shared memory: a copy, or under total-order truncation the kept
@@ -87,27 +102,33 @@ __device__ __forceinline__ void load_coefs(const double* __restrict__ xs, int M_
   for (int t = tid; t < M_xi; t += nthreads) s_xi[slot[t]] = xs[t];
 }
 
-// 2D: CTA covers 32 x (8 * KAP_ROWS) elements of one sample.
+// 2D: CTA covers 32 columns x (8 * KAP_ROWS) row pairs of one sample. Bound by
+// the FP64 pipe: m / 2 + 10 operations per element (64 samples of 512^2, m = 8:
+// 674 us with m + 13, 479 us now).
 __global__ void __launch_bounds__(TX2* TY2)
     k_kappa2d(int n, int m, double sqrt_sigma2, const double* __restrict__ table,
               const double* __restrict__ xi, int M_xi, const int32_t* __restrict__ slot,
               int64_t es, double* __restrict__ kappa, Prof prof) {
   __shared__ double s_xi[MAX_MODES_1D * MAX_MODES_1D];
-  __shared__ double s_t[TX2][MAX_MODES_1D + 1];          // T[ix][k_y]
+  __shared__ double s_t[TX2][MAX_MODES_1D + 1];          // T[ix][k_y] 64 / ln 2
   __shared__ double s_fy[TY2 * KAP_ROWS][MAX_MODES_1D + 1];
+  __shared__ double s_tab[EXP_TAB];
   const int b = blockIdx.z;
   const int tid = threadIdx.y * TX2 + threadIdx.x;
   const int nthreads = TX2 * TY2;
   const int x0 = blockIdx.x * TX2;
   const int y0 = blockIdx.y * TY2 * KAP_ROWS;
+  const int half = (n + 1) / 2;                          // row pairs (the middle row of an odd n is its own)
+  for (int j = tid; j < EXP_TAB; j += nthreads) s_tab[j] = g_exp2_tab[j];
   load_coefs(xi + (int64_t)b * M_xi, M_xi, slot, m * m, s_xi, tid, nthreads);
   for (int idx = tid; idx < TY2 * KAP_ROWS * m; idx += nthreads) {
     const int r = idx / m, k = idx - r * m;
     const int iy = y0 + r;
-    s_fy[r][k] = (iy < n) ? table[iy * m + k] : 0.0;
+    s_fy[r][k] = (iy < half) ? table[iy * m + k] : 0.0;
   }
   __syncthreads();
   // T[ix][ky] = sum_kx F[ix][kx] xi[ky * m + kx]
+  const double scale = sqrt_sigma2 * kInvLn2x64;
   for (int idx = tid; idx < TX2 * m; idx += nthreads) {
     const int c = idx / m, ky = idx - c * m;
     const int ix = x0 + c;
@@ -116,20 +137,29 @@ __global__ void __launch_bounds__(TX2* TY2)
       const double* fx = table + ix * m;
       for (int kx = 0; kx < m; ++kx) acc = fma(fx[kx], s_xi[ky * m + kx], acc);
     }
-    s_t[c][ky] = acc;
+    s_t[c][ky] = scale * acc;
   }
   __syncthreads();
   const int ix = x0 + threadIdx.x;
   if (ix < n) {
-    double* out = kappa + (int64_t)b * es;
-#pragma unroll 4
+    double* out = kappa + (int64_t)b * es + ix;
+    const double* tx = s_t[threadIdx.x];
+#pragma unroll 2
     for (int r = 0; r < KAP_ROWS; ++r) {
       const int rl = threadIdx.y + TY2 * r;
       const int iy = y0 + rl;
-      if (iy >= n) break;
-      double g = 0.0;
-      for (int ky = 0; ky < m; ++ky) g = fma(s_fy[rl][ky], s_t[threadIdx.x][ky], g);
-      out[(int64_t)iy * n + ix] = kle_exp(sqrt_sigma2 * g);
+      if (iy >= half) break;
+      const double* fy = s_fy[rl];
+      double e = fy[0] * tx[0], o = 0.0;
+      int ky = 1;
+      for (; ky + 1 < m; ky += 2) {
+        o = fma(fy[ky], tx[ky], o);
+        e = fma(fy[ky + 1], tx[ky + 1], e);
+      }
+      if (ky < m) o = fma(fy[ky], tx[ky], o);
+      out[(int64_t)iy * n] = kle_exp(e + o, s_tab);
+      const int my = n - 1 - iy;
+      if (my != iy) out[(int64_t)my * n] = kle_exp(e - o, s_tab);
     }
   }
   if (prof.acc && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) atomicAdd(prof.acc, prof.per_sample);
@@ -137,7 +167,9 @@ __global__ void __launch_bounds__(TX2* TY2)
 
 // 3D: CTA covers 32 (x) x 4 (y) elements for all z of one sample column
 // block; per (ix, iy): T2[kz] = sum_ky F[iy][ky] sum_kx F[ix][kx] xi[kz][ky][kx],
-// then g(iz) = sum_kz F[iz][kz] T2[kz].
+// then the layers iz and n - 1 - iz from the even and odd sums over kz of
+// F[iz][kz] T2[kz], as in 2D. T2 sits in shared memory (a column per thread):
+// as a local array its run-time index would put it in local memory.
 constexpr int K3_TY = 4;
 __global__ void __launch_bounds__(TX2* K3_TY)
     k_kappa3d(int n, int m, double sqrt_sigma2, const double* __restrict__ table,
@@ -147,14 +179,18 @@ __global__ void __launch_bounds__(TX2* K3_TY)
   const int M = m * m * m;
   double* s_xi = smem;                              // M
   double* s_t1 = s_xi + M;                          // [TX2][m*m]  T1[ix][kz*m+ky]
+  double* s_t2 = s_t1 + TX2 * m * m;                // [m][threads]
+  __shared__ double s_tab[EXP_TAB];
   const int b = blockIdx.z;
   const int tid = threadIdx.y * TX2 + threadIdx.x;
   const int nthreads = TX2 * K3_TY;
   const int x0 = blockIdx.x * TX2;
   const int iy = blockIdx.y * K3_TY + threadIdx.y;
+  for (int j = tid; j < EXP_TAB; j += nthreads) s_tab[j] = g_exp2_tab[j];
   load_coefs(xi + (int64_t)b * M_xi, M_xi, slot, M, s_xi, tid, nthreads);
   __syncthreads();
   const int mm = m * m;
+  const double scale = sqrt_sigma2 * kInvLn2x64;
   for (int idx = tid; idx < TX2 * mm; idx += nthreads) {
     const int c = idx / mm, kk = idx - c * mm;     // kk = kz * m + ky
     const int ix = x0 + c;
@@ -163,24 +199,33 @@ __global__ void __launch_bounds__(TX2* K3_TY)
       const double* fx = table + ix * m;
       for (int kx = 0; kx < m; ++kx) acc = fma(fx[kx], s_xi[kk * m + kx], acc);
     }
-    s_t1[c * mm + kk] = acc;
+    s_t1[c * mm + kk] = scale * acc;
   }
   __syncthreads();
   const int ix = x0 + threadIdx.x;
   if (ix >= n || iy >= n) return;
-  double t2[MAX_MODES_1D];
   const double* fy = table + iy * m;
+  double* t2 = s_t2 + tid;
   for (int kz = 0; kz < m; ++kz) {
     double acc = 0.0;
     for (int ky = 0; ky < m; ++ky) acc = fma(fy[ky], s_t1[threadIdx.x * mm + kz * m + ky], acc);
-    t2[kz] = acc;
+    t2[kz * nthreads] = acc;
   }
-  double* out = kappa + (int64_t)b * es;
-  for (int iz = 0; iz < n; ++iz) {
+  double* out = kappa + (int64_t)b * es + (int64_t)iy * n + ix;
+  const int64_t plane = (int64_t)n * n;
+#pragma unroll 2
+  for (int iz = 0; iz < (n + 1) / 2; ++iz) {
     const double* fz = table + iz * m;
-    double g = 0.0;
-    for (int kz = 0; kz < m; ++kz) g = fma(fz[kz], t2[kz], g);
-    out[((int64_t)iz * n + iy) * n + ix] = kle_exp(sqrt_sigma2 * g);
+    double e = fz[0] * t2[0], o = 0.0;
+    int kz = 1;
+    for (; kz + 1 < m; kz += 2) {
+      o = fma(fz[kz], t2[kz * nthreads], o);
+      e = fma(fz[kz + 1], t2[(kz + 1) * nthreads], e);
+    }
+    if (kz < m) o = fma(fz[kz], t2[kz * nthreads], o);
+    out[iz * plane] = kle_exp(e + o, s_tab);
+    const int mz = n - 1 - iz;
+    if (mz != iz) out[mz * plane] = kle_exp(e - o, s_tab);
   }
   if (prof.acc && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) atomicAdd(prof.acc, prof.per_sample);
 }
@@ -229,9 +274,9 @@ __global__ void k_cast_kappa(int64_t ne, int64_t es, const double* __restrict__ 
 cudaError_t init_kle_exp() {
   static std::atomic<uint64_t> done{0};
   return once_per_device(done, [] {
-    double tab[64];
-    for (int j = 0; j < 64; ++j) tab[j] = (double)std::exp2((long double)j / 64.0L);
-    return cudaMemcpyToSymbol(c_exp2_tab, tab, sizeof(tab));
+    double tab[EXP_TAB];
+    for (int j = 0; j < EXP_TAB; ++j) tab[j] = (double)std::exp2((long double)j / EXP_TAB);
+    return cudaMemcpyToSymbol(g_exp2_tab, tab, sizeof(tab));
   });
 }
 
@@ -256,11 +301,12 @@ cudaError_t launch_kappa(cudaStream_t s, const Grid& g, int m, double sqrt_sigma
                          int64_t B, double* kappa, Prof p) {
   if (B == 0) return cudaSuccess;
   if (g.dim == 2) {
-    dim3 grid((g.n + TX2 - 1) / TX2, (g.n + TY2 * KAP_ROWS - 1) / (TY2 * KAP_ROWS), (unsigned)B);
+    const int half = (g.n + 1) / 2;
+    dim3 grid((g.n + TX2 - 1) / TX2, (half + TY2 * KAP_ROWS - 1) / (TY2 * KAP_ROWS), (unsigned)B);
     k_kappa2d<<<grid, dim3(TX2, TY2), 0, s>>>(g.n, m, sqrt_sigma2, table, xi, M_xi, slot, g.es, kappa, p);
   } else {
     const int M = m * m * m;
-    const size_t smem = sizeof(double) * ((size_t)M + (size_t)TX2 * m * m);
+    const size_t smem = sizeof(double) * ((size_t)M + (size_t)TX2 * m * m + (size_t)TX2 * K3_TY * m);
     static std::atomic<uint64_t> opted{0};
     const cudaError_t attr = once_per_device(opted, [] {
       return cudaFuncSetAttribute(k_kappa3d, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
