@@ -590,12 +590,10 @@ def roofline_of(res, peaks, fp64_alu, dim=2, fp64_probe=None):
 
 def kle_compare(m, wl, stream, peaks, batch=None, reps=10):
     """The KLE contraction of one coupled batch of the finest mesh: the FP64
-    sum-factorised kernel (mlmc_kappa, the kappa of the FP64 residual) and the
-    tensor-core kernel (mlmc_kappa32, split BF16 on tcgen05, the FP32 kappa of
-    the inner solves), each timed with CUDA events on the plan's stream.
-    Tensor roofline: the dense contraction's flops 2 ne M B and the flops the
-    MMAs issue (three BF16 products on tiles padded to 128 elements x 64
-    modes x 16 samples) against the measured BF16 peak."""
+    kernel (mlmc_kappa, the kappa of the FP64 residual) and the FP32 one
+    (mlmc_kappa32, the FP32 kappa of the inner solves), both sum-factorised,
+    each timed with CUDA events on the plan's stream; the FP32 kernel is bound
+    by its store, 4 bytes per element, against the measured copy bandwidth."""
     import torch
     L = wl["levels"] - 1
     n = wl["n0"] << L
@@ -614,7 +612,7 @@ def kle_compare(m, wl, stream, peaks, batch=None, reps=10):
             k32 = torch.empty(B * es, dtype=torch.float32, device="cuda")
             for name, fn in (("fp64_sum_factorised",
                               lambda: plan.kappa(L, xi.data_ptr(), B, k64.data_ptr())),
-                             ("tensor_cores_split_bf16",
+                             ("fp32_sum_factorised",
                               lambda: plan.kappa32(L, xi.data_ptr(), B, k32.data_ptr()))):
                 fn()
                 torch.cuda.synchronize()
@@ -626,18 +624,13 @@ def kle_compare(m, wl, stream, peaks, batch=None, reps=10):
                 e1.record(stream)
                 torch.cuda.synchronize()
                 res[name] = {"ms": e0.elapsed_time(e1) / reps}
-    dense = 2.0 * ne * M * B
-    issued = 3 * 2.0 * ((ne + 127) // 128 * 128) * ((M + 63) // 64 * 64) * ((min(B, 256) + 15) // 16 * 16) \
-        * ((B + 255) // 256)
-    t = res["tensor_cores_split_bf16"]["ms"] / 1e3
-    peak = peaks.get("bf16_tflops")
-    tens = {"bound": "tensor", "achieved": round(issued / t / 1e12, 2), "unit": "TFLOP/s",
-            "dense_contraction_tflops": round(dense / t / 1e12, 2),
-            "peak": peak, "peak_source": "measured (MEASURED_PEAKS.json bf16_tflops)" if peak else None,
-            "frac": round(issued / t / 1e12 / peak, 4) if peak else None,
-            "kappa32_write_gbs": round(4.0 * ne * B / t / 1e9, 1)}
-    res["tensor_roofline"] = tens
-    res["faster"] = min(("fp64_sum_factorised", "tensor_cores_split_bf16"), key=lambda k: res[k]["ms"])
+    t = res["fp32_sum_factorised"]["ms"] / 1e3
+    peak = peaks.get("hbm_gbs")
+    res["fp32_roofline"] = {"bound": "hbm", "achieved": round(4.0 * ne * B / t / 1e9, 1), "unit": "GB/s",
+                            "peak": peak,
+                            "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peak else None,
+                            "frac": round(4.0 * ne * B / t / 1e9 / peak, 4) if peak else None}
+    res["faster"] = min(("fp64_sum_factorised", "fp32_sum_factorised"), key=lambda k: res[k]["ms"])
     return res
 
 
@@ -693,7 +686,7 @@ def bench_ours(args):
     pk_path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(pk_path):
         peaks = json.load(open(pk_path))
-    # the mixed form with its FP32 kappa from the tensor cores (kle_tensor = 1)
+    # the mixed form with its FP32 kappa made directly (kle_tensor = 1)
     kle_tc = None
     if not args.single_form and "mixed" in forms:
         cfg = m.config_from_workload(wl, precision="mixed", kle_tensor=1)
@@ -729,7 +722,7 @@ def bench_ours(args):
             "kappa_share": kle_tc["shares"].get("kappa"), "autotune": kle_tc["tune"]}
     if rank == 0:
         names = {"fp64": "plain FP64", "mixed": "mixed: FP32 inner PCG + FP64 refinement",
-                 "mixed+kle_tensor": "mixed, FP32 kappa from the tensor-core KLE"}
+                 "mixed+kle_tensor": "mixed, FP32 kappa made from the KLE coefficients"}
         line = {"metric": "coupled DOF-solves/s", "value": value, "unit": "coupled DOF-solves/s",
                 "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
                 "ms_per_step": ms / args.steps, "time_to_eps_s": ms / args.steps / 1e3,

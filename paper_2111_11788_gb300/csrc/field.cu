@@ -90,16 +90,17 @@ constexpr int KAP_ROWS = 4;
 // The sample's KLE coefficients in the full tensor layout (m^dim entries) in
 // shared memory: a copy, or under total-order truncation the kept
 // coefficients scattered to their full-basis slots and zeros elsewhere.
+template <class V>
 __device__ __forceinline__ void load_coefs(const double* __restrict__ xs, int M_xi,
                                            const int32_t* __restrict__ slot, int M_full,
-                                           double* s_xi, int tid, int nthreads) {
+                                           V* s_xi, int tid, int nthreads) {
   if (!slot) {
-    for (int k = tid; k < M_full; k += nthreads) s_xi[k] = xs[k];
+    for (int k = tid; k < M_full; k += nthreads) s_xi[k] = (V)xs[k];
     return;
   }
-  for (int k = tid; k < M_full; k += nthreads) s_xi[k] = 0.0;
+  for (int k = tid; k < M_full; k += nthreads) s_xi[k] = V(0);
   __syncthreads();
-  for (int t = tid; t < M_xi; t += nthreads) s_xi[slot[t]] = xs[t];
+  for (int t = tid; t < M_xi; t += nthreads) s_xi[slot[t]] = (V)xs[t];
 }
 
 // 2D: CTA covers 32 columns x (8 * KAP_ROWS) row pairs of one sample. Bound by
@@ -230,6 +231,157 @@ __global__ void __launch_bounds__(TX2* K3_TY)
   if (prof.acc && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) atomicAdd(prof.acc, prof.per_sample);
 }
 
+// kappa in FP32 for the mixed form's inner solves: the same sum factorisation
+// and mirrored pairs with FP32 sums, kappa32 = 2^t by the hardware
+// approximation (ex2.approx, relative error about 2^-22), t = x / ln 2. A
+// thread takes K32_P consecutive row (layer) pairs of one column at a time,
+// so a mode costs it one load of the column's contraction and one 16-byte
+// load of the axis table for K32_P multiply-adds. Bound by the store of kappa32
+// (4 B per element): a dense contraction over all M modes, on the tensor cores
+// or not, does M multiply-adds per element where this does m / 2 + 1.
+constexpr int K32_P = 4;
+constexpr int K32_Y = 8;          // warps per CTA
+constexpr int K32_ROWS = 128;     // 2D: row pairs per CTA
+
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// even and odd sums over the modes of K32_P consecutive pairs: t the column's
+// contraction (stride ts), f the axis table, f[k * fs + pair]
+__device__ __forceinline__ void even_odd(int m, const float* t, int ts, const float* f, int fs, float (&e)[K32_P],
+                                         float (&o)[K32_P]) {
+#pragma unroll
+  for (int q = 0; q < K32_P; ++q) e[q] = o[q] = 0.f;
+  auto add = [&](int k, float (&a)[K32_P]) {
+    const float tv = t[k * ts];
+    const float4 fv = *reinterpret_cast<const float4*>(f + k * fs);
+    a[0] = fmaf(fv.x, tv, a[0]);
+    a[1] = fmaf(fv.y, tv, a[1]);
+    a[2] = fmaf(fv.z, tv, a[2]);
+    a[3] = fmaf(fv.w, tv, a[3]);
+  };
+  int k = 0;
+  for (; k + 1 < m; k += 2) {
+    add(k, e);
+    add(k + 1, o);
+  }
+  if (k < m) add(k, e);
+}
+
+__global__ void __launch_bounds__(TX2* K32_Y)
+    k_kappa32_2d(int n, int m, float scale, const double* __restrict__ table, const double* __restrict__ xi, int M_xi,
+                 const int32_t* __restrict__ slot, int64_t es, float* __restrict__ kappa) {
+  __shared__ float s_xi[MAX_MODES_1D * MAX_MODES_1D];
+  __shared__ float s_t[TX2][MAX_MODES_1D + 1];                      // T[ix][k_y] / ln 2
+  __shared__ __align__(16) float s_f[MAX_MODES_1D][K32_ROWS];       // F[iy][k_y]
+  __shared__ float s_fx[TX2][MAX_MODES_1D + 1];                     // F[ix][k_x]
+  const int b = blockIdx.z, nthreads = TX2 * K32_Y;
+  const int tid = threadIdx.y * TX2 + threadIdx.x;
+  const int x0 = blockIdx.x * TX2, y0 = blockIdx.y * K32_ROWS, half = (n + 1) / 2;
+  load_coefs(xi + (int64_t)b * M_xi, M_xi, slot, m * m, s_xi, tid, nthreads);
+  for (int idx = tid; idx < K32_ROWS * m; idx += nthreads) {
+    const int r = idx / m, k = idx - r * m;
+    s_f[k][r] = y0 + r < half ? (float)table[(y0 + r) * m + k] : 0.f;
+  }
+  for (int idx = tid; idx < TX2 * m; idx += nthreads) {
+    const int c = idx / m, k = idx - c * m;
+    s_fx[c][k] = x0 + c < n ? (float)table[(x0 + c) * m + k] : 0.f;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < TX2 * m; idx += nthreads) {
+    const int c = idx / m, ky = idx - c * m;
+    float acc = 0.f;
+    for (int kx = 0; kx < m; ++kx) acc = fmaf(s_fx[c][kx], s_xi[ky * m + kx], acc);
+    s_t[c][ky] = scale * acc;
+  }
+  __syncthreads();
+  const int ix = x0 + threadIdx.x;
+  if (ix >= n) return;
+  float* out = kappa + (int64_t)b * es + ix;
+  for (int p = threadIdx.y * K32_P; p < K32_ROWS && y0 + p < half; p += K32_Y * K32_P) {
+    float e[K32_P], o[K32_P];
+    even_odd(m, s_t[threadIdx.x], 1, &s_f[0][p], K32_ROWS, e, o);
+#pragma unroll
+    for (int q = 0; q < K32_P; ++q) {
+      const int iy = y0 + p + q, my = n - 1 - iy;
+      if (iy < half) {
+        out[(int64_t)iy * n] = ex2_approx(e[q] + o[q]);
+        if (my != iy) out[(int64_t)my * n] = ex2_approx(e[q] - o[q]);
+      }
+    }
+  }
+}
+
+// half (rounded up to K32_P) of the layers' table in shared memory
+inline int k32_half(int n) { return ((n + 1) / 2 + K32_P - 1) / K32_P * K32_P; }
+inline size_t k32_smem3(int n, int m) {
+  return sizeof(float) * ((size_t)m * k32_half(n) + (size_t)m * m * m + (size_t)TX2 * (m * m + 1) +
+                          (size_t)m * TX2 * K32_Y + (size_t)TX2 * (m + 1) + (size_t)K32_Y * m);
+}
+
+__global__ void __launch_bounds__(TX2* K32_Y)
+    k_kappa32_3d(int n, int m, int fs, float scale, const double* __restrict__ table, const double* __restrict__ xi,
+                 int M_xi, const int32_t* __restrict__ slot, int64_t es, float* __restrict__ kappa) {
+  extern __shared__ __align__(16) float sm32[];
+  const int mm = m * m, M = mm * m, half = (n + 1) / 2, nthreads = TX2 * K32_Y;
+  float* s_f = sm32;                       // [m][fs] F[iz][k_z] of the first half of the layers
+  float* s_xi = s_f + m * fs;              // [M]
+  float* s_t1 = s_xi + M;                  // [TX2][mm + 1] T1[ix][k_z m + k_y] / ln 2
+  float* s_t2 = s_t1 + TX2 * (mm + 1);     // [m][threads] T2[k_z] of each column
+  float* s_fx = s_t2 + m * nthreads;       // [TX2][m + 1] F[ix][k_x]
+  float* s_fy = s_fx + TX2 * (m + 1);      // [K32_Y][m] F[iy][k_y]
+  const int b = blockIdx.z;
+  const int tid = threadIdx.y * TX2 + threadIdx.x;
+  const int x0 = blockIdx.x * TX2, iy = blockIdx.y * K32_Y + threadIdx.y;
+  load_coefs(xi + (int64_t)b * M_xi, M_xi, slot, M, s_xi, tid, nthreads);
+  for (int idx = tid; idx < fs * m; idx += nthreads) {
+    const int r = idx / m, k = idx - r * m;
+    s_f[k * fs + r] = r < half ? (float)table[r * m + k] : 0.f;
+  }
+  for (int idx = tid; idx < TX2 * m; idx += nthreads) {
+    const int c = idx / m, k = idx - c * m;
+    s_fx[c * (m + 1) + k] = x0 + c < n ? (float)table[(x0 + c) * m + k] : 0.f;
+  }
+  for (int idx = tid; idx < K32_Y * m; idx += nthreads) {
+    const int r = idx / m, k = idx - r * m, y = blockIdx.y * K32_Y + r;
+    s_fy[r * m + k] = y < n ? (float)table[y * m + k] : 0.f;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < TX2 * mm; idx += nthreads) {
+    const int c = idx & (TX2 - 1), kk = idx / TX2;   // lanes along x: the coefficient is a broadcast
+    float acc = 0.f;
+    for (int kx = 0; kx < m; ++kx) acc = fmaf(s_fx[c * (m + 1) + kx], s_xi[kk * m + kx], acc);
+    s_t1[c * (mm + 1) + kk] = scale * acc;
+  }
+  __syncthreads();
+  const int ix = x0 + threadIdx.x;
+  if (ix >= n || iy >= n) return;
+  float* t2 = s_t2 + tid;
+  const float* t1 = s_t1 + threadIdx.x * (mm + 1);
+  for (int kz = 0; kz < m; ++kz) {
+    float acc = 0.f;
+    for (int ky = 0; ky < m; ++ky) acc = fmaf(s_fy[threadIdx.y * m + ky], t1[kz * m + ky], acc);
+    t2[kz * nthreads] = acc;
+  }
+  float* out = kappa + (int64_t)b * es + (int64_t)iy * n + ix;
+  const int64_t plane = (int64_t)n * n;
+  for (int p = 0; p < half; p += K32_P) {
+    float e[K32_P], o[K32_P];
+    even_odd(m, t2, nthreads, s_f + p, fs, e, o);
+#pragma unroll
+    for (int q = 0; q < K32_P; ++q) {
+      const int iz = p + q, mz = n - 1 - iz;
+      if (iz < half) {
+        out[iz * plane] = ex2_approx(e[q] + o[q]);
+        if (mz != iz) out[mz * plane] = ex2_approx(e[q] - o[q]);
+      }
+    }
+  }
+}
+
 template <class T>
 __global__ void k_coarsen2d(int nc, const T* __restrict__ kf, T* __restrict__ kc,
                             int64_t esf, int64_t esc, Prof prof) {
@@ -315,6 +467,27 @@ cudaError_t launch_kappa(cudaStream_t s, const Grid& g, int m, double sqrt_sigma
     dim3 grid((g.n + TX2 - 1) / TX2, (g.n + K3_TY - 1) / K3_TY, (unsigned)B);
     k_kappa3d<<<grid, dim3(TX2, K3_TY), smem, s>>>(g.n, m, sqrt_sigma2, table, xi, M_xi, slot, g.es,
                                                    kappa, p);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_kappa32(cudaStream_t s, const Grid& g, int m, double sqrt_sigma2, const double* table,
+                           const double* xi, int M_xi, const int32_t* slot, int64_t B, float* kappa32) {
+  if (B == 0) return cudaSuccess;
+  const float scale = (float)(sqrt_sigma2 * 1.4426950408889634074);   // 1 / ln 2
+  const dim3 block(TX2, K32_Y);
+  if (g.dim == 2) {
+    const dim3 grid((g.n + TX2 - 1) / TX2, ((g.n + 1) / 2 + K32_ROWS - 1) / K32_ROWS, (unsigned)B);
+    k_kappa32_2d<<<grid, block, 0, s>>>(g.n, m, scale, table, xi, M_xi, slot, g.es, kappa32);
+  } else {
+    static std::atomic<uint64_t> opted{0};
+    const cudaError_t attr = once_per_device(opted, [] {
+      return cudaFuncSetAttribute(k_kappa32_3d, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    });
+    if (attr != cudaSuccess) return attr;
+    const dim3 grid((g.n + TX2 - 1) / TX2, (g.n + K32_Y - 1) / K32_Y, (unsigned)B);
+    k_kappa32_3d<<<grid, block, k32_smem3(g.n, m), s>>>(g.n, m, k32_half(g.n), scale, table, xi, M_xi, slot, g.es,
+                                                        kappa32);
   }
   return cudaGetLastError();
 }

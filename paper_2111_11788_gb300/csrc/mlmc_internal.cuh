@@ -172,11 +172,9 @@ cudaError_t launch_coarsen(cudaStream_t s, const Grid& fine, const Grid& coarse,
 // kappa32 = (float) kappa64, element arrays.
 // the table of the FP64 exp of the kappa kernels, once per device (before any capture)
 cudaError_t init_kle_exp();
-// kappa32 = exp(Phi xi) on the tensor cores (split BF16, FP32 accumulation); M kept modes
-cudaError_t launch_kappa32_tc(cudaStream_t s, const Grid& g, int m, double sqrt_sigma2, const double* table,
-                              const double* xi, int M, const int32_t* slot, int64_t B, float* kappa32);
-// bounded waits of the tensor-core KLE kernel that gave up since the last call (resets the count)
-cudaError_t take_tc_timeouts(cudaStream_t s, unsigned* out);
+// kappa32 = exp(Phi xi) with FP32 sums
+cudaError_t launch_kappa32(cudaStream_t s, const Grid& g, int m, double sqrt_sigma2, const double* table,
+                           const double* xi, int M_xi, const int32_t* slot, int64_t B, float* kappa32);
 cudaError_t launch_cast_kappa(cudaStream_t s, const Grid& g, const double* k64, float* k32,
                               int64_t B);
 

@@ -146,7 +146,7 @@ struct MixedWs {
   double* r;
   double* kap64;
   double* coef64;   // operator data of the outer FP64 residual: 2D coefficients, 3D kappa sums
-  const double* xi_tc;  // KLE coefficients: the FP32 kappa from the tensor cores (else the cast)
+  const double* xi32;   // KLE coefficients: the FP32 kappa made from them (else the cast)
   Scalars outer;
   int32_t* outer_count;
   int32_t* outer_it;
@@ -160,7 +160,7 @@ void carve_mixed(Carve& c, const MeshInfo& mi, int64_t B, MixedWs& w) {
   w.r = c.take<double>(B * g0.ns);
   w.kap64 = c.take<double>(B * g0.es);
   w.coef64 = g0.dim == 2 ? c.take<double>(B * (3 * g0.ns + g0.es)) : c.take<double>(B * 4 * g0.ns);
-  w.xi_tc = nullptr;
+  w.xi32 = nullptr;
   w.outer.gamma = w.outer.delta = w.outer.alpha = w.outer.beta = nullptr;
   w.outer.rho = c.take<double>(B);
   w.outer.tol = c.take<double>(B);
@@ -210,7 +210,7 @@ void carve_coupled(Carve& c, const MeshInfo& mi, int M, int64_t B, bool mixed, i
   if (mixed) {
     carve_mixed(c, mi, B, w.mx);
     w.kap = w.mx.kap64;
-    w.mx.xi_tc = w.xi;   // used when the plan takes its FP32 kappa from the tensor cores
+    w.mx.xi32 = w.xi;   // used when the plan makes its FP32 kappa itself (kle_tensor)
     w.mx.outer_execs = execs ? execs + 2 * side : nullptr;
     w.mx.in.execs = execs ? execs + 2 * side + 1 : nullptr;
   } else {
@@ -291,7 +291,6 @@ struct mlmc_plan_s {
   double ms[NUM_KERNELS] = {0};
   int64_t kl[NUM_KERNELS] = {0};
   int64_t launches = 0;
-  bool tc_used = false;           // the tensor-core KLE kernel has run on this plan
   bool zw_used = false;   // mlmc_apply32 ran the 3D FP32 z-march (bounded waits to check)
   // graph-captured solves, keyed by (form, mesh, batch, workspace) and the
   // arrays they bake in (kappa, solution, QoI, iteration counts, guess)
@@ -998,11 +997,6 @@ mlmc_status settle_graph_launches(mlmc_plan p) {
     CK(d3::take_wait_timeouts(p->stream, &timeouts));
     if (timeouts) return MLMC_ERR_TIMEOUT;
   }
-  if (p->tc_used) {
-    unsigned timeouts = 0;
-    CK(take_tc_timeouts(p->stream, &timeouts));
-    if (timeouts) return MLMC_ERR_TIMEOUT;
-  }
   for (const GraphRec* r : p->pending_graphs) {
     p->launches += r->n_static;
     for (const auto& lp : r->loops) {
@@ -1132,9 +1126,9 @@ mlmc_status mixed_setup(mlmc_plan p, const MeshInfo& mi, MixedWs& w, int64_t B, 
   cudaStream_t s = p->stream;
   const mlmc_config& c = p->cfg;
   const Grid& g0 = mi.g[0];
-  if (w.xi_tc && c.kle_tensor) {
+  if (w.xi32 && c.kle_tensor) {
     CK(run(p, KID_KAPPA, [&] {
-      return launch_kappa32_tc(s, g0, c.modes_per_dim, p->sqrt_sigma2, mi.table, w.xi_tc, p->M, p->d_slot, B,
+      return launch_kappa32(s, g0, c.modes_per_dim, p->sqrt_sigma2, mi.table, w.xi32, p->M, p->d_slot, B,
                                w.in.kap[0]);
     }));
   } else {
@@ -1527,7 +1521,7 @@ mlmc_status issue_level_group(mlmc_plan p, int level, const std::vector<int64_t>
       o += cnt;
       xo += cnt * q->M;
     }
-    if (mixed) w.mx.xi_tc = nullptr;   // members' coefficients differ in number: kappa32 by the cast
+    if (mixed) w.mx.xi32 = nullptr;   // members' coefficients differ in number: kappa32 by the cast
     double* qd = side == 0 ? w.qf : w.qc;
     int32_t* itd = side == 0 ? w.itf : w.itc;
     const Guess gs = guess_views(p, level, side, mixed, w);
@@ -1801,7 +1795,6 @@ mlmc_status mlmc_plan_create(const mlmc_config* cfg, void* stream, mlmc_plan* ou
   mlmc_plan p = new mlmc_plan_s();
   p->cfg = *cfg;
   p->stream = (cudaStream_t)stream;
-  p->tc_used = cfg->kle_tensor && cfg->precision == MLMC_MIXED;
   const int m = cfg->modes_per_dim;
   p->M = (int)coef_count(cfg);
   p->sqrt_sigma2 = std::sqrt(cfg->sigma2);
@@ -2038,11 +2031,10 @@ mlmc_status mlmc_kappa32(mlmc_plan p, int mesh, const double* xi, int64_t count,
   if (!p || mesh < 0 || mesh >= p->cfg.n_levels || count < 0 || (count > 0 && (!xi || !kappa32)))
     return MLMC_ERR_INVALID;
   const MeshInfo& mi = p->meshes[mesh];
-  p->tc_used = true;
   for (int64_t off = 0; off < count; off += 65535) {
     const int64_t B = std::min<int64_t>(65535, count - off);
     CK(run(p, KID_KAPPA, [&] {
-      return launch_kappa32_tc(p->stream, mi.g[0], p->cfg.modes_per_dim, p->sqrt_sigma2, mi.table,
+      return launch_kappa32(p->stream, mi.g[0], p->cfg.modes_per_dim, p->sqrt_sigma2, mi.table,
                                xi + off * p->M, p->M, p->d_slot, B, kappa32 + off * mi.g[0].es);
     }));
   }

@@ -1,11 +1,13 @@
-"""The field kernels on mirrored element pairs: kappa (FP64) against the oracle's dense exp(Phi xi) where the pairing has its edges: odd
+"""The field kernels on mirrored element pairs: kappa (FP64) and kappa32 (FP32)
+against the oracle's dense exp(Phi xi) where the pairing has its edges: odd
 meshes (the middle row or layer is its own partner), meshes of less than a
 tile, one mode, odd numbers of modes, a truncated basis, and fields beyond the
 normal range of exp.
 
 Bound: with A the sum of |Phi_k xi_k| over the modes, an axis-by-axis sum of m
 terms per axis with tables a few ulps off rounds to within dim (m + 6) + 8
-units of A; kappa adds a few ulps of its own."""
+units of A; kappa adds a few ulps of its own (FP32: 2^-21 for the hardware's
+power of two)."""
 import numpy as np
 import pytest
 
@@ -32,10 +34,12 @@ def fields(m, dim, n, mpd, order, sigma2, xi):
     es, ne, count = m.elem_stride(dim, n), n ** dim, xi.shape[0]
     x = torch.from_numpy(np.ascontiguousarray(xi)).cuda()
     k64 = torch.full((count, es), -1.0, dtype=torch.float64, device="cuda")
+    k32 = torch.full((count, es), -1.0, dtype=torch.float32, device="cuda")
     with m.Plan(cfg, torch.cuda.current_stream().cuda_stream) as plan:
         plan.kappa(0, x.data_ptr(), count, k64.data_ptr())
+        plan.kappa32(0, x.data_ptr(), count, k32.data_ptr())
         torch.cuda.synchronize()
-    return k64.cpu().numpy()[:, :ne]
+    return k64.cpu().numpy()[:, :ne], k32.cpu().numpy()[:, :ne].astype(np.float64)
 
 
 @pytest.mark.parametrize("dim,n,mpd,order", [
@@ -49,9 +53,10 @@ def test_fields_against_oracle(m, dim, n, mpd, order):
     xi = rng.standard_normal((3, M))
     phi = kle.phi_matrix(dim, n, 0.2, 1.5, mpd, kept)
     ref, A = np.exp(xi @ phi.T), np.abs(xi) @ np.abs(phi).T
-    k64 = fields(m, dim, n, mpd, order, 1.5, xi)
+    k64, k32 = fields(m, dim, n, mpd, order, 1.5, xi)
     units = dim * (mpd + 6) + 8
     assert np.all(np.abs(k64 - ref) <= (units * A + 8) * 2.0 ** -53 * ref)
+    assert np.all(np.abs(k32 - ref) <= ((units * A + 8) * 2.0 ** -24 + 2.0 ** -21) * ref)
 
 
 def test_fields_beyond_the_range_of_exp(m):
@@ -61,7 +66,7 @@ def test_fields_beyond_the_range_of_exp(m):
     top = 1000.0 / phi.max()
     xi = np.array([[top], [-top], [0.7 * top], [-0.7 * top], [np.nan]])
     x = xi @ phi.T
-    k64 = fields(m, 2, n, 1, -1, 1.0, xi)
+    k64, _ = fields(m, 2, n, 1, -1, 1.0, xi)
     with np.errstate(over="ignore", under="ignore"):
         ref = np.exp(x)
     assert np.isnan(k64[4]).all()
