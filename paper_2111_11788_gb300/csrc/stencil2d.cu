@@ -28,6 +28,7 @@
 // write one FP64 partial per warp (stencil kernels, g.tiles_s per sample)
 // or per CTA (flat kernels, g.tiles_f per sample), summed in a fixed order
 // by k_finalize.
+#include "guess.cuh"
 #include "mlmc_internal.cuh"
 
 namespace mlmc {
@@ -1228,8 +1229,42 @@ __global__ void __launch_bounds__(SBLOCK) k_restrict2s(Grid gc, int64_t nsf, con
   }
 }
 
-// Nested initial guess: x = P uc, the coarse-mesh solution interpolated
-// bilinearly to the fine mesh (0 on the boundary), one thread per node.
+// Nested initial guess by cubic interpolation of the coarse-mesh solution, on
+// warp strips: a lane walks one coarse column down GUESS_ROWS fine rows with
+// the four coarse values around its row in registers, and takes its
+// neighbours' for the odd columns: 3 FP64 operations per node.
+constexpr int GUESS_ROWS = 32;
+__global__ void __launch_bounds__(SBLOCK) k_guess2(Grid g, int64_t nsc, const double* __restrict__ Uc,
+                                                   double* __restrict__ X, const int32_t* __restrict__ active,
+                                                   Prof prof) {
+  const int64_t b = blockIdx.z;
+  if (!active[b]) return;
+  const int n = g.n, N1 = n + 1, nc = n / 2, C1 = nc + 1, lane = threadIdx.x & 31;
+  const int I0 = (blockIdx.x * SWARPS + (threadIdx.x >> 5)) * GUESS_COLS;
+  if (I0 > nc) return;   // the whole strip lies beyond the row
+  const int I = I0 - GUESS_HALO + lane;
+  const bool in = I >= 0 && I <= nc;
+  const bool out = in && lane >= GUESS_HALO && lane < GUESS_HALO + GUESS_COLS;
+  const double* uc = Uc + b * nsc + (in ? I : 0);
+  double* x = X + b * g.ns;
+  auto at = [&](int J) { return in ? __ldg(uc + J * C1) : 0.0; };
+  const int y0 = blockIdx.y * GUESS_ROWS, y1 = min(y0 + GUESS_ROWS, N1);
+  CubicWindow w;
+  w.start(y0, nc, at);
+  for (int j = y0; j < y1; ++j) {
+    w.advance(j, nc, at);
+    const bool rin = j > 0 && j < n;
+    const double v = w.value(j, nc), o = guess_odd(I, nc, v);
+    if (out) {
+      x[(int64_t)j * N1 + 2 * I] = rin && I > 0 && I < nc ? v : 0.0;
+      if (I < nc) x[(int64_t)j * N1 + 2 * I + 1] = rin ? o : 0.0;
+    }
+  }
+  if (prof.acc && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(prof.acc, prof.per_sample);
+}
+
+// The same by bilinear interpolation (coarse meshes of less than
+// CUBIC_MIN_CELLS cells per side), one thread per node.
 __global__ void __launch_bounds__(FLAT_THREADS) k_prolong_guess2(Grid g, int64_t nsc,
                                                                  const double* __restrict__ Uc,
                                                                  double* __restrict__ X,
@@ -1427,7 +1462,12 @@ namespace d2 {
 
 cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, const double* uc,
                           double* x, const int32_t* active, int64_t B, Prof p) {
-  k_prolong_guess2<<<fgrid(g, B), FLAT_THREADS, 0, s>>>(g, coarse.ns, uc, x, active, p);
+  if (coarse.n >= CUBIC_MIN_CELLS)
+    k_guess2<<<dim3((unsigned)((coarse.n + SWARPS * GUESS_COLS) / (SWARPS * GUESS_COLS)),
+                    (unsigned)((g.n + GUESS_ROWS) / GUESS_ROWS), (unsigned)B),
+               SBLOCK, 0, s>>>(g, coarse.ns, uc, x, active, p);
+  else
+    k_prolong_guess2<<<fgrid(g, B), FLAT_THREADS, 0, s>>>(g, coarse.ns, uc, x, active, p);
   return cudaGetLastError();
 }
 
