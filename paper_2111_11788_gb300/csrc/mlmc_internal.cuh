@@ -116,11 +116,18 @@ constexpr int MAX_BOTTOM = 8;
 template <class T>
 struct BottomLevels {
   int L;                       // fused levels (the last is the coarsest, n = 2)
+  int cycles;                  // 2D: 2 = a second cycle on the residual of the first
   Grid g[MAX_BOTTOM];
   const T* kap[MAX_BOTTOM];
   const T* coef[MAX_BOTTOM];
   const T* w[MAX_BOTTOM];
 };
+// 2D meshes of at least this many cells per side run the fused levels twice
+// per V-cycle: a V-cycle's convergence falls behind the two-grid rate (0.077
+// against 0.024 per iteration) by what its coarse levels leave unsolved, and
+// here the second cycle costs a fused launch beside stencils on grids 64
+// and more times larger: one CG iteration less of eight on 512^2 and 1024^2.
+constexpr int BOTTOM_TWICE_N2 = 512;
 // largest grid (cells per side) whose level is fused: 2D, 3D
 constexpr int BOTTOM_MAX_N2 = 64;
 constexpr int BOTTOM_MAX_N3 = 16;

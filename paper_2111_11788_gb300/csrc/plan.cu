@@ -713,6 +713,7 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
   if (fuse) {
     BottomLevels<T> lv{};
     lv.L = K - k0;
+    lv.cycles = g0.dim == 2 && g0.n >= BOTTOM_TWICE_N2 ? 2 : 1;
     double bytes = 2 * nodes_of(mi.g[k0]);
     for (int l = 0; l < lv.L; ++l) {
       lv.g[l] = mi.g[k0 + l];

@@ -1325,7 +1325,8 @@ __device__ __forceinline__ T prolong2_s(const T* ec, int nc, int i, int j) {
 // same steps and arithmetic as k_mgpre2, k_restrict2, k_coarse2 and
 // k_mgpost2 (C: FP64 coefficient form with residuals accumulated from b;
 // else kappa form), with a barrier between steps instead of a launch.
-// Operator data, W and kappa are read from global memory (cached).
+// Operator data, W and kappa are read from global memory (cached). With
+// lv.cycles 2 the levels run a second time on the residual of the first.
 template <class T, bool C>
 __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom2(BottomLevels<T> lv, const T* __restrict__ Bv,
                                                             T* __restrict__ Out,
@@ -1380,6 +1381,20 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom2(BottomLevels<T> lv, 
     for (int i = tid; i < N1 * N1; i += BOTTOM_THREADS) b[i] = src[i];
   }
   __syncthreads();
+  T* acc = base(L);   // two cycles: the first one's result
+  for (int cyc = 0; cyc < lv.cycles; ++cyc) {
+  if (cyc > 0) {
+    // the next cycle's right-hand side: the residual of the first cycle's result
+    const int n = lv.g[0].n, N1 = n + 1, nn = N1 * N1;
+    T* b = base(0);
+    const T* t = b + 2 * nn;
+    for (int i = tid; i < nn; i += BOTTOM_THREADS) {
+      const int j = i / N1, c = i - j * N1;
+      acc[i] = t[i];
+      if (interior2(n, c, j)) b[i] = resid(0, t, c, j, b[i]);
+    }
+    __syncthreads();
+  }
   // down: e = W b, r1 = b - A e, b_{l+1} = R r1
   for (int l = 0; l < L - 1; ++l) {
     const int n = lv.g[l].n, N1 = n + 1, nn = N1 * N1;
@@ -1445,11 +1460,12 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom2(BottomLevels<T> lv, 
     }
     __syncthreads();
   }
+  }
   {
     const int N1 = lv.g[0].n + 1;
     const T* t = base(0) + 2 * N1 * N1;
     T* dst = Out + smp * lv.g[0].ns;
-    for (int i = tid; i < N1 * N1; i += BOTTOM_THREADS) dst[i] = t[i];
+    for (int i = tid; i < N1 * N1; i += BOTTOM_THREADS) dst[i] = lv.cycles > 1 ? acc[i] + t[i] : t[i];
   }
   if (prof.acc && tid == 0) atomicAdd(prof.acc, prof.per_sample);
 }
@@ -1633,11 +1649,13 @@ cudaError_t mg_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b, T* 
     return cudaErrorInvalidValue;
   size_t smem = 0;
   for (int l = 0; l < lv.L; ++l) smem += 3 * (size_t)(lv.g[l].n + 1) * (lv.g[l].n + 1) * sizeof(T);
+  if (lv.cycles > 1) smem += (size_t)(lv.g[0].n + 1) * (lv.g[0].n + 1) * sizeof(T);
   // opt in (once per device) to the shared memory of the largest fused chain (64^2 .. 2^2)
   static std::atomic<uint64_t> opted{0};
   const cudaError_t attr = once_per_device(opted, [] {
     size_t most = 0;
     for (int n = BOTTOM_MAX_N2; n >= 2; n /= 2) most += 3 * (size_t)(n + 1) * (n + 1) * sizeof(T);
+    most += (size_t)(BOTTOM_MAX_N2 + 1) * (BOTTOM_MAX_N2 + 1) * sizeof(T);   // two cycles
     cudaError_t e1 = cudaFuncSetAttribute(k_bottom2<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     cudaError_t e2 = cudaFuncSetAttribute(k_bottom2<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     return e1 != cudaSuccess ? e1 : e2;

@@ -444,3 +444,20 @@ def test_apply_is_the_same_on_every_strip_height(m, n, count):
     torch.cuda.synchronize()
     got = many.reshape(count, ns)[:, :nn]
     assert torch.equal(got, one[:nn].expand(count, nn))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_solve_parity_with_two_bottom_cycles(m, precision):
+    """512^2: the fused multigrid levels run twice per V-cycle from this size on."""
+    n = 512
+    cfg = m.config(dim=2, n_levels=1, coarse_cells=n, solver="gmg", rtol=1e-11, precision=precision)
+    kap = random_element_field(2, n, 1, seed=3, spread=0.5)
+    u, q, it = dev(m.node_stride(2, n)), dev(1), dev(1, torch.int32)
+    with m.Plan(cfg, stream()) as plan:
+        kd = elem_arrays_to_device(m, 2, n, kap)
+        plan.solve(0, kd.data_ptr(), 1, u.data_ptr(), q.data_ptr(), it.data_ptr())
+    ref = fem.solve(fem.assemble_fast(2, n, kap[0]), fem.load_vector(2, n), 2)
+    qref = fem.qoi_weights(2, n) @ ref
+    got = fem.from_node_grid(2, n, u.cpu().numpy()[:(n + 1) ** 2])
+    assert int(it[0]) > 0 and abs(float(q[0]) - qref) <= RTOL_Q * abs(qref)
+    assert np.max(np.abs(got - ref)) <= 1e-7 * np.max(np.abs(ref))
