@@ -768,6 +768,7 @@ constexpr int ZSTAGES = 4;   // planes in flight: the current one and ZSTAGES - 
 // and combined pairwise into the field once the plane has arrived.
 struct LdXf {   // x
   static constexpr int kArrays = 1;
+  static constexpr bool kCoarse = false;
   const float* a0;
   int64_t ns;
   __device__ void bind(int64_t b) { a0 += b * ns; }
@@ -779,6 +780,7 @@ struct LdXf {   // x
 
 struct LdPupdf {   // z + beta p (beta == 0: z)
   static constexpr int kArrays = 2;
+  static constexpr bool kCoarse = false;
   const float* z;
   const float* pold;
   const double* beta;
@@ -799,6 +801,7 @@ struct LdPupdf {   // z + beta p (beta == 0: z)
 
 struct LdWbf {   // omega D^-1 b
   static constexpr int kArrays = 2;
+  static constexpr bool kCoarse = false;
   const float* W;
   const float* Bv;
   int64_t ns;
@@ -1022,9 +1025,9 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3f(Grid g, const float* __res
 // k_zm3w is k_zm3f with its planes staged by the copy engine instead of by
 // per-element cp.async, for the meshes with n in {32, 64, 128, 256}: a CTA
 // covers the full width of the mesh (n threads across x, one column each)
-// and R = 256 RT / n node rows, RT rows per thread (RT = 2: the CTAs per
-// sample are those of the 32 x 16 tiles; RT = 4: half as many, each
-// covering two of them), so the halo slab of a plane (rows ty0 - 1 ..
+// and R = 256 RT / n node rows, RT = 2 rows per thread (the CTAs per sample
+// are those of the 32 x 16 tiles; k_zm3n takes four rows per thread and half
+// as many CTAs), so the halo slab of a plane (rows ty0 - 1 ..
 // ty0 + R, every column) is one contiguous range of a node array; the kappa
 // slab (rows ty0 - 1 .. ty0 + R - 1) is one contiguous range of an element
 // array. Each plane of each array is then ONE asynchronous bulk copy
@@ -1038,7 +1041,7 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3f(Grid g, const float* __res
 // and the layers -1 and n) may be stale; planes 0 and n are not copied, and
 // the boundary nodes of the field (rows, columns and planes 0 and n) are
 // read as 0 by the threads next to them, whatever the array holds there.
-// A thread's RT rows are RT / 2 float2 pairs of consecutive rows. Waits are
+// A thread's two rows are one float2 pair. Waits are
 // bounded: a wait that gives up counts a timeout in g_zt_timeouts (read by
 // the host at its sync points), lets the copies still in flight land
 // (bounded again) and ends the CTA.
@@ -1097,14 +1100,13 @@ __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
 
-template <class Ld, class Epi, int RT>
-__global__ void __launch_bounds__(ZTHREADS, RT == 2 ? 3 : 2) k_zm3w(Grid g, const float* __restrict__ Kap, Ld ld,
+template <class Ld, class Epi>
+__global__ void __launch_bounds__(ZTHREADS, 3) k_zm3w(Grid g, const float* __restrict__ Kap, Ld ld,
                                                                    const int32_t* __restrict__ active, Epi epi,
                                                                    double* __restrict__ part, Prof prof) {
   static_assert(!Epi::kRes, "the FP32 z-march hands A x to its epilogues");
-  static_assert(RT == 2 || RT == 4, "two or four rows per thread");
   constexpr int NA = Ld::kArrays;
-  constexpr int NP = RT / 2;   // float2 row pairs per thread
+  constexpr int RT = 2, NP = 1;   // rows and float2 row pairs per thread
   const int64_t b = blockIdx.y;
   if (active && !active[b]) return;
   extern __shared__ __align__(16) float zw_smem[];
@@ -1339,8 +1341,6 @@ __global__ void __launch_bounds__(ZTHREADS, RT == 2 ? 3 : 2) k_zm3w(Grid g, cons
     return;
   }
   if (part) {
-    // the partial sits where the first 32 x 16 tile of this CTA's rows puts
-    // it; the other tiles it covers (RT = 4) get 0
     double v = warp_sum3((double)dot);
     if ((tid & 31) == 0) s_w[tid >> 5] = v;
     __syncthreads();
@@ -1348,17 +1348,358 @@ __global__ void __launch_bounds__(ZTHREADS, RT == 2 ? 3 : 2) k_zm3w(Grid g, cons
       double r = 0.0;
 #pragma unroll
       for (int w = 0; w < ZTHREADS / 32; ++w) r += s_w[w];
-      const int R2 = zw_rows(n, 2);
-      double* pt = part + (int64_t)blockIdx.y * g.tiles_s + (int64_t)zq * (n / R2) + ty0 / R2;
-      pt[0] = r;
+      part[(int64_t)blockIdx.y * g.tiles_s + blockIdx.x] = r;
+    }
+  }
+  prof_tick3(prof);
+}
+
+// k_zm3n: the z-march of k_zm3w with four rows per thread and the mesh's width a
+// compile-time constant, so that every shared-memory and node offset inside a
+// plane is an immediate. Bound by instruction issue: the form with a run-time
+// width spent 109 warp instructions per 32 nodes on the FP32 operator (63% of
+// the issue slots, 159 us for 16 samples of 128^3), 33 of which are its
+// arithmetic. What else changed: the two rows of a pair are 2 apart (rows
+// jr0 + q and jr0 + q + 2 of output pair q), so the pairs of one output pair
+// serve the other's neighbours and need no register moves; boundary values of
+// a field that may be nonzero there are cleared in shared memory once per
+// plane by the few threads next to the barrier instead of being selected
+// away by every thread; the slab's shift is carried (a plane has an odd number
+// of nodes, N1^2 = 1 mod 4: one float further each plane); the epilogue's own
+// inputs are read without a test, boundary nodes included. 109 us then, 55% of
+// the copy bandwidth (registers allow two CTAs per SM).
+template <int N, class Ld, class Epi>
+__global__ void __launch_bounds__(ZTHREADS, 2) k_zm3n(Grid g, const float* __restrict__ Kap, Ld ld,
+                                                      const int32_t* __restrict__ active, Epi epi,
+                                                      double* __restrict__ part, Prof prof) {
+  static_assert(!Epi::kRes, "the FP32 z-march hands A x to its epilogues");
+  constexpr int NA = Ld::kArrays, RT = 4;
+  constexpr int N1 = N + 1, P = N1 * N1, KPn = N * N;
+  constexpr int R = zw_rows(N, RT), VS = zw_vslot(N, RT), KS = zw_kslot(N, RT), SS = NA * VS + KS;
+  static_assert((P & 3) == 1, "the slab's shift grows by one float a plane");
+  const int64_t b = blockIdx.y;
+  if (active && !active[b]) return;
+  extern __shared__ __align__(16) float zw_smem[];
+  float* ring = zw_smem;                                              // ZW_S slots of SS floats
+  unsigned long long* sbar = reinterpret_cast<unsigned long long*>(zw_smem + ZW_S * SS);
+  __shared__ double s_w[ZTHREADS / 32];
+  // P e_c: the coarse rows under a slab, interpolated along z to plane p, in
+  // scz[p & 1] (rows J0 .. J0 + CR - 1 of CC nodes)
+  constexpr int C1 = N / 2 + 1, CR = R / 2 + 2, CE = Ld::kCoarse ? CR * C1 : 1;
+  constexpr int CPT = (CE + ZTHREADS - 1) / ZTHREADS;
+  float* scz = reinterpret_cast<float*>(sbar + ZW_S);
+  constexpr int tyn = N / R;
+  const int zq = blockIdx.x / tyn;
+  const int ty0 = (blockIdx.x - zq * tyn) * R;
+  const int z0 = zq * g.zc, z1 = min(z0 + g.zc, N1);
+  const int i = threadIdx.x, tid = threadIdx.y * N + i;
+  const float* __restrict__ kp_ = Kap + b * g.es;
+  ld.bind(b);
+  epi.bind(b);
+  for (int e = tid; e < ZW_S * SS / 4; e += ZTHREADS)
+    reinterpret_cast<float4*>(ring)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const unsigned bar0 = (unsigned)__cvta_generic_to_shared(sbar);
+  const unsigned ring0 = (unsigned)__cvta_generic_to_shared(ring);
+  if (tid == 0) {
 #pragma unroll
-      for (int k = 1; k < NP; ++k) pt[k] = 0.0;
+    for (int s = 0; s < ZW_S; ++s) mbar_init(bar0 + 8u * s, 1u);
+    fence_mbar_init();
+  }
+  fence_proxy_async_smem();
+  __syncthreads();
+
+  // slabs: node rows ylo..yhi of a plane, kappa rows kylo..ty0 + R - 1 of a layer
+  const int ylo = max(ty0 - 1, 0), yhi = min(ty0 + R, N), r0 = ylo - ty0 + 1;
+  const int kylo = max(ty0 - 1, 0), kr0 = kylo - ty0 + 1;
+  const unsigned kbytes = 4u * (unsigned)((ty0 + R - kylo) * N);
+  auto voff = [&](int pp) { return ((pp * P + ylo * N1) - r0 * N1) & 3; };
+  // stage plane pp (field) and layer pp (kappa) into slot st: one bulk copy per array
+  auto issue = [&](int pp, int st) {
+    if (tid != 0) return;
+    const bool pv = pp >= 1 && pp < N, pk = pp >= 0 && pp < N;
+    const unsigned bar = bar0 + 8u * st;
+    const int G0 = pp * P + ylo * N1, G1 = pp * P + (yhi + 1) * N1;
+    const int Ga = G0 & ~3, Gb = (G1 + 3) & ~3;
+    const unsigned vbytes = 4u * (unsigned)(Gb - Ga);
+    mbar_arrive_tx(bar, (pv ? NA * vbytes : 0u) + (pk ? kbytes : 0u));
+    if (pv) {
+      const int dst = 4 + voff(pp) + r0 * N1 - (G0 - Ga);
+#pragma unroll
+      for (int a = 0; a < NA; ++a)
+        bulk_g2s(ring0 + 4u * (unsigned)(st * SS + a * VS + dst), ld.src(a) + Ga, vbytes, bar);
+    }
+    if (pk)
+      bulk_g2s(ring0 + 4u * (unsigned)(st * SS + NA * VS + 4 + kr0 * N), kp_ + (pp * KPn + kylo * N), kbytes, bar);
+  };
+
+  int p = z0 - 1;
+  unsigned pend = 0;   // slots with copies issued and not yet waited for
+#pragma unroll
+  for (int j = 0; j < ZW_S - 1; ++j)
+    if (p + j <= z1) {
+      issue(p + j, j);
+      pend |= 1u << j;
+    }
+
+  float cn[CPT];   // this thread's entries of the next plane's coarse rows
+  const int J0 = ty0 / 2 - 1;
+  auto coarse_fetch = [&](int pp) {
+    if constexpr (Ld::kCoarse) {
+      const bool pv = pp >= 1 && pp < N;
+#pragma unroll
+      for (int q = 0; q < CPT; ++q) {
+        const int e = tid + q * ZTHREADS, J = J0 + e / C1;
+        float v = 0.f;
+        if (pv && e < CE && J >= 0 && J < C1) {
+          const float* c = ld.ec + ((pp >> 1) * C1 + J) * C1 + e % C1;
+          v = __ldg(c);
+          if (pp & 1) v = 0.5f * (v + __ldg(c + C1 * C1));
+        }
+        cn[q] = v;
+      }
+    }
+  };
+  auto coarse_store = [&](int pp) {
+    if constexpr (Ld::kCoarse) {
+#pragma unroll
+      for (int q = 0; q < CPT; ++q)
+        if (tid + q * ZTHREADS < CE) scz[(pp & 1) * CE + tid + q * ZTHREADS] = cn[q];
+    }
+  };
+  if constexpr (Ld::kCoarse) {   // the first plane's rows, the second's on their way
+    coarse_fetch(p);
+    coarse_store(p);
+    coarse_fetch(p + 1);
+    __syncthreads();
+  }
+
+  const int jr0 = ty0 + RT * (int)threadIdx.y;   // this thread's rows jr0 .. jr0 + 3
+  const bool ci = i >= 1, c0 = ci && jr0 > 0;    // interior column; interior node of row jr0
+  const bool ex = i == N - 1, ey = jr0 + RT == N;
+  const float c3s = (float)g.c3, c12s = (float)g.c12;
+  const float2 c3 = make_float2(c3s, c3s), mc12 = make_float2(-c12s, -c12s);
+  const float2 z2 = make_float2(0.f, 0.f);
+  // output pair q: rows jr0 + q and jr0 + q + 2. As in k_zm3f: U unscaled
+  // couplings and D diagonal part of the output of plane p - 1, Nn couplings
+  // of the output of plane p with plane p - 1; of the kappa layer below, the
+  // element pairs (kb), their sums along x (Xb), along y (Yb) and of four (Sb)
+  float2 U[2], D[2], Nn[2], vc[2], kb[3][2], Xb[3], Yb[2][2], Sb[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) U[q] = D[q] = Nn[q] = vc[q] = Sb[q] = Yb[q][0] = Yb[q][1] = z2;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) kb[k][0] = kb[k][1] = Xb[k] = z2;
+  typename Epi::Pre pre[RT];
+  float dot = 0.0f;
+  const float* vthr = ring + 4 + RT * (int)threadIdx.y * N1 + i - 1;            // + shift: row jr0 - 1, column i - 1
+  const float* kthr = ring + NA * VS + 4 + RT * (int)threadIdx.y * N + i - 1;   // row jr0 - 1, element i - 1
+  const int o0 = jr0 * N1 + i;
+  int sh = voff(p);
+  int st = 0;
+  unsigned par = 0;    // phase parity of each slot's next completion
+  bool timed_out = false;
+#pragma unroll 2
+  for (; p <= z1; ++p) {
+    const bool landed = mbar_wait(bar0 + 8u * st, (par >> st) & 1u);
+    if (landed) {
+      pend &= ~(1u << st);
+      par ^= 1u << st;
+    }
+    float* slot = ring + st * SS;
+    if (landed && p >= 1 && p < N) {
+      if constexpr (Ld::kCoarse) {   // W b + P e_c (0 on the boundary, as W, b and e_c are)
+        const float* cz = scz + (p & 1) * CE + (i >> 1);
+        const int ox = i & 1;
+#pragma unroll
+        for (int rr = (int)threadIdx.y; rr < R + 2; rr += ZTHREADS / N) {
+          const int jj = rr + 1;                     // fine row ty0 - 1 + rr = 2 J0 + jj
+          const float* c = cz + (jj >> 1) * C1;
+          float h = c[0] + c[ox];                    // twice the value along x
+          h = (jj & 1) ? 0.25f * (h + (c[C1] + c[C1 + ox])) : 0.5f * h;
+          float* e = slot + 4 + sh + rr * N1 + i;
+          e[0] = fmaf(e[0], e[VS], h);
+        }
+      } else if constexpr (NA > 1) {   // combine the arrays into the field (both are 0 on the boundary)
+        for (int e = tid; e < VS; e += ZTHREADS) slot[e] = ld.combine1(slot[e], slot[VS + e]);
+      } else {                  // clear the field's boundary columns and rows
+        float* row = slot + 4 + sh;
+        if (tid < R + 2) row[tid * N1] = row[tid * N1 + N] = 0.f;
+        if (ty0 == 0 && threadIdx.y == 0) row[N1 + i] = 0.f;
+        if (ty0 + R == N && threadIdx.y == 0) row[(R + 1) * N1 + i] = 0.f;
+      }
+    }
+    coarse_store(p + 1);
+    fence_proxy_async_smem();       // this thread's shared-memory writes before later copies
+    // plane p complete; the slot of plane p - 1 is free (or a wait gave up:
+    // every thread leaves the loop together)
+    if (__syncthreads_or(!landed)) {
+      timed_out = true;
+      break;
+    }
+    coarse_fetch(p + 2);
+    if (p + ZW_S - 1 <= z1) {
+      const int sn = (st + ZW_S - 1) % ZW_S;
+      issue(p + ZW_S - 1, sn);
+      pend |= 1u << sn;
+    }
+    typename Epi::Pre nxt[RT];
+    if (p >= z0 && p < z1 && p >= 1 && p < N) {
+#pragma unroll
+      for (int r = 0; r < RT; ++r) nxt[r] = epi.load(p * P + o0 + r * N1);
+    }
+    // node row pairs (jr0 - 1 + k, jr0 + 1 + k), element row pairs likewise
+    float2 v[4][3], ka[3][2];
+    if (p >= 1 && p < N) {
+      const float* sv = vthr + st * SS + sh;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) v[k][dx] = make_float2(sv[k * N1 + dx], sv[(k + 2) * N1 + dx]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) v[k][dx] = z2;
+    }
+    {
+      const float* sk = kthr + st * SS;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int a = 0; a < 2; ++a) ka[k][a] = make_float2(sk[k * N + a], sk[(k + 2) * N + a]);
+    }
+    float2 Xa[3], Ya[2][2], Sa[2], ks[3][2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      Xa[k] = add2(ka[k][0], ka[k][1]);
+      ks[k][0] = add2(kb[k][0], ka[k][0]);
+      ks[k][1] = add2(kb[k][1], ka[k][1]);
+    }
+    const int m = p - 1;
+    const bool mi = m >= 1 && m < N;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      Ya[q][0] = add2(ka[q][0], ka[q + 1][0]);
+      Ya[q][1] = add2(ka[q][1], ka[q + 1][1]);
+      Sa[q] = add2(Xa[q], Xa[q + 1]);
+      const float2 *v0 = v[q], *v1 = v[q + 1], *v2 = v[q + 2];
+      // outputs of plane p - 1 are complete: couplings with plane p across layer p - 1
+      float2 u = fma2(Yb[q][0], v1[0], U[q]);
+      u = fma2(Yb[q][1], v1[2], u);
+      u = fma2(Xb[q], v0[1], u);
+      u = fma2(Xb[q + 1], v2[1], u);
+      u = fma2(kb[q][0], v0[0], u);
+      u = fma2(kb[q][1], v0[2], u);
+      u = fma2(kb[q + 1][0], v2[0], u);
+      u = fma2(kb[q + 1][1], v2[2], u);
+      const float2 done = fma2(mc12, u, mul2(c3, D[q]));
+      if (m >= z0) {
+        const int o = m * P + o0;
+        dot += epi(o + q * N1, (q ? ci : c0) && mi, done.x, vc[q].x, pre[q]);
+        dot += epi(o + (q + 2) * N1, ci && mi, done.y, vc[q].y, pre[q + 2]);
+      }
+      // output p: couplings with plane p - 1 and the in-plane diagonal edges
+      u = fma2(ks[q][0], v0[0], Nn[q]);
+      u = fma2(ks[q][1], v0[2], u);
+      u = fma2(ks[q + 1][0], v2[0], u);
+      U[q] = fma2(ks[q + 1][1], v2[2], u);
+      D[q] = mul2(add2(Sb[q], Sa[q]), v1[1]);
+      // output p + 1: couplings with plane p across layer p
+      u = mul2(Ya[q][0], v1[0]);
+      u = fma2(Ya[q][1], v1[2], u);
+      u = fma2(Xa[q], v0[1], u);
+      u = fma2(Xa[q + 1], v2[1], u);
+      u = fma2(ka[q][0], v0[0], u);
+      u = fma2(ka[q][1], v0[2], u);
+      u = fma2(ka[q + 1][0], v2[0], u);
+      Nn[q] = fma2(ka[q + 1][1], v2[2], u);
+      vc[q] = v1[1];
+    }
+    if (m >= z0) {   // boundary nodes beyond the tile's last column and row
+      const int o = m * P + o0;
+      if (ex) {
+#pragma unroll
+        for (int r = 0; r < RT; ++r) epi.zero(o + r * N1 + 1);
+      }
+      if (ey) {
+        epi.zero(o + RT * N1);
+        if (ex) epi.zero(o + RT * N1 + 1);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      kb[k][0] = ka[k][0];
+      kb[k][1] = ka[k][1];
+      Xb[k] = Xa[k];
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      Yb[q][0] = Ya[q][0];
+      Yb[q][1] = Ya[q][1];
+      Sb[q] = Sa[q];
+    }
+#pragma unroll
+    for (int r = 0; r < RT; ++r) pre[r] = nxt[r];
+    st = (st + 1) % ZW_S;
+    sh = (sh + 1) & 3;
+  }
+  if (timed_out) {
+    // record the timeout, let the copies still in flight land (bounded), end the CTA
+    if (tid == 0) atomicAdd(&g_zt_timeouts, 1u);
+    for (int s2 = 0; s2 < ZW_S; ++s2)
+      if (pend & (1u << s2)) mbar_wait(bar0 + 8u * s2, (par >> s2) & 1u);
+    return;
+  }
+  if (part) {
+    // the partial sits where the first 32 x 16 tile of this CTA's rows puts
+    // it; the other tile it covers gets 0
+    double v = warp_sum3((double)dot);
+    if ((tid & 31) == 0) s_w[tid >> 5] = v;
+    __syncthreads();
+    if (tid == 0) {
+      double r = 0.0;
+#pragma unroll
+      for (int w = 0; w < ZTHREADS / 32; ++w) r += s_w[w];
+      constexpr int R2 = zw_rows(N, 2);
+      double* pt = part + (int64_t)blockIdx.y * g.tiles_s + (int64_t)zq * (N / R2) + ty0 / R2;
+      pt[0] = r;
+      pt[1] = 0.0;
     }
   }
   prof_tick3(prof);
 }
 
 inline dim3 gridz(const Grid& g, int64_t B) { return dim3((unsigned)g.zx, (unsigned)B, 1); }
+
+// Full-width tiles staged by bulk copies: n in 32..256 and the partials'
+// layout of whole tiles (every grid of make_grid with stencil_tile 0 or 2).
+inline bool zm_wide(const Grid& g) {
+  return g.zt != 1 && zw_mesh(g.n) && g.ns % 4 == 0 && g.es % 4 == 0 &&
+         (g.zx == (int64_t)(g.n / zw_rows(g.n, 2)) * ((g.n + 1 + g.zc - 1) / g.zc));
+}
+
+template <int N, class LP, class Epi>
+inline void launch_zm3n_at(cudaStream_t s, const Grid& g, int64_t B, const float* kappa, const LP& lp,
+                           const int32_t* active, const Epi& epi, double* part, Prof p) {
+  constexpr int NA = LP::kArrays, R = zw_rows(N, 4);
+  // up to 76 KB of ring and coarse rows per CTA (opt-in above 48 KB)
+  constexpr int smem = (int)sizeof(float) * ZW_S * (NA * zw_vslot(N, 4) + zw_kslot(N, 4)) + 8 * ZW_S +
+                       (LP::kCoarse ? (int)sizeof(float) * 2 * (R / 2 + 2) * (N / 2 + 1) : 0);
+  static std::atomic<uint64_t> opted{0};
+  if (once_per_device(opted, [] {
+        return cudaFuncSetAttribute(k_zm3n<N, LP, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      }) != cudaSuccess)
+    return;   // the launcher's cudaGetLastError reports it
+  k_zm3n<N, LP, Epi><<<dim3((unsigned)(g.zx / 2), (unsigned)B, 1), dim3(N, ZTHREADS / N, 1), smem, s>>>(
+      g, kappa, lp, active, epi, part, p);
+}
+template <class LP, class Epi>
+inline void launch_zm3n(cudaStream_t s, const Grid& g, int64_t B, const float* kappa, const LP& lp,
+                        const int32_t* active, const Epi& epi, double* part, Prof p) {
+  if (g.n == 32) launch_zm3n_at<32>(s, g, B, kappa, lp, active, epi, part, p);
+  else if (g.n == 64) launch_zm3n_at<64>(s, g, B, kappa, lp, active, epi, part, p);
+  else if (g.n == 128) launch_zm3n_at<128>(s, g, B, kappa, lp, active, epi, part, p);
+  else launch_zm3n_at<256>(s, g, B, kappa, lp, active, epi, part, p);
+}
 
 // The z-march launch of an epilogue: the paired FP32 kernel for float.
 template <class T, class Ld, class Epi>
@@ -1377,24 +1718,13 @@ inline void launch_zm3(cudaStream_t s, const Grid& g, int64_t B, const T* kappa,
     const typename LP::type lp = LP::make(ld);
     // bulk-copy staging: full-width tiles (n in 32..256), 16-byte aligned arrays;
     // stencil_tile 0: four rows per thread, 2: two rows per thread
-    if (g.zt != 1 && zw_mesh(g.n) && lp.aligned16() && ((uintptr_t)kappa & 15) == 0 && g.ns % 4 == 0 &&
-        g.es % 4 == 0 && (g.zx == (int64_t)(g.n / zw_rows(g.n, 2)) * ((g.n + 1 + g.zc - 1) / g.zc))) {
+    if (zm_wide(g) && lp.aligned16() && ((uintptr_t)kappa & 15) == 0) {
       constexpr int NA = LP::type::kArrays;
-      // four rows per thread: up to 71 KB of ring per CTA (opt-in above 48 KB)
-      static std::atomic<uint64_t> opted{0};
-      const bool four = g.zt == 0 && once_per_device(opted, [] {
-                                       return cudaFuncSetAttribute(k_zm3w<typename LP::type, Epi, 4>,
-                                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                                   96 * 1024);
-                                     }) == cudaSuccess;
-      if (four) {
-        const size_t smem = sizeof(float) * ZW_S * (NA * zw_vslot(g.n, 4) + zw_kslot(g.n, 4)) + 8 * ZW_S;
-        k_zm3w<typename LP::type, Epi, 4><<<dim3((unsigned)(g.zx / 2), (unsigned)B, 1),
-                                           dim3(g.n, ZTHREADS / g.n, 1), smem, s>>>(g, kappa, lp, active, epi,
-                                                                                   part, p);
+      if (g.zt == 0) {
+        launch_zm3n(s, g, B, kappa, lp, active, epi, part, p);
       } else {
         const size_t smem = sizeof(float) * ZW_S * (NA * zw_vslot(g.n, 2) + zw_kslot(g.n, 2)) + 8 * ZW_S;
-        k_zm3w<typename LP::type, Epi, 2><<<gridz(g, B), dim3(g.n, ZTHREADS / g.n, 1), smem, s>>>(
+        k_zm3w<typename LP::type, Epi><<<gridz(g, B), dim3(g.n, ZTHREADS / g.n, 1), smem, s>>>(
             g, kappa, lp, active, epi, part, p);
       }
     }

@@ -127,3 +127,20 @@ def test_apply32_3d_128_against_fp64_operator(m, tile):
         full = y[s].reshape((n + 1,) * 3)
         assert np.all(full[0] == 0) and np.all(full[-1] == 0)
         assert np.all(full[:, 0] == 0) and np.all(full[:, :, -1] == 0)
+
+
+@pytest.mark.parametrize("n", [32, 64, 128, 256])
+def test_apply32_3d_ignores_boundary_entries(m, n):
+    """Full-width tiles of every width: boundary entries of x, NaN among them, do not reach any output."""
+    x, k = inputs(3, n, 1, seed=n)
+    g = x.reshape(n + 1, n + 1, n + 1)
+    clean, dirty = g.copy(), g.copy()
+    for a in range(3):
+        for end in (0, n):
+            at = [slice(None)] * 3
+            at[a] = end
+            clean[tuple(at)] = 0.0
+            dirty[tuple(at)] = np.nan
+    want = apply32(m, 3, n, clean.reshape(1, -1), k)
+    for got, ref in zip(apply32(m, 3, n, dirty.reshape(1, -1), k), want):
+        assert np.isfinite(ref).all() and np.array_equal(got, ref)
