@@ -815,6 +815,25 @@ struct LdWbf {   // omega D^-1 b
   bool aligned16() const { return (((uintptr_t)W | (uintptr_t)Bv) & 15) == 0; }
 };
 
+// The corrected iterate omega D^-1 b + P e_c (k_zm3n only): W and b are staged
+// and the pre-smoothed iterate formed from them again, P e_c added from coarse
+// rows kept in shared memory. Neither the iterate nor its sum with the
+// correction is stored by a pass of its own.
+struct LdPostf {
+  static constexpr int kArrays = 2;
+  static constexpr bool kCoarse = true;
+  const float* W;
+  const float* Bv;
+  const float* ec;
+  int64_t ns, nsc;
+  __device__ void bind(int64_t b) {
+    W += b * ns;
+    Bv += b * ns;
+    ec += b * nsc;
+  }
+  __device__ const float* src(int k) const { return k ? Bv : W; }
+};
+
 template <class Ld>
 struct LdPaired;
 template <>
@@ -2174,7 +2193,11 @@ cudaError_t pcg_pq(cudaStream_t s, const Grid& g, const T* kappa, const T* z, co
 template <class T>
 cudaError_t mg_pre(cudaStream_t s, const Grid& g, const T* kappa, const T* w, const T* b, T* e, T* r1,
                    const int32_t* active, int64_t B, Prof p, const T* ks) {
-  launch_zm3<T>(s, g, B, kappa, LdWb<T>{w, b, g.ns}, active, EpiMgRes<T>{b, r1, e, g.ns}, nullptr, p, ks);
+  // FP32 levels whose post-smoother forms e = W b again do not store it (mg_post's test)
+  const bool keep = !(sizeof(T) == 4 && zm_wide(g) && g.zt == 0 &&
+                      (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) == 0);
+  launch_zm3<T>(s, g, B, kappa, LdWb<T>{w, b, g.ns}, active, EpiMgRes<T>{b, r1, keep ? e : nullptr, g.ns}, nullptr, p,
+                ks);
   return cudaGetLastError();
 }
 template <class T>
@@ -2195,6 +2218,14 @@ template <class T>
 cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* kappa, const T* w,
                     const T* b, const T* e, const T* ec, T* out, T* tmp, const int32_t* active,
                     double* part, int64_t B, Prof p, const T* ks) {
+  if constexpr (std::is_same<T, float>::value) {
+    // one kernel (the arrays are a plan's, 256-byte aligned; e is not read)
+    if (zm_wide(g) && g.zt == 0 && (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) == 0) {
+      launch_zm3n(s, g, B, kappa, LdPostf{w, b, ec, g.ns, coarse.ns}, active, EpiMgPost<float>{w, b, out, g.ns}, part,
+                  p);
+      return cudaGetLastError();
+    }
+  }
   k_prolong3<T><<<prolong3_grid(g, B), dim3(32, 8, 1), 0, s>>>(g, coarse.ns, e, ec, tmp, active,
                                                                  Prof{nullptr, 0.0});
   launch_zm3<T>(s, g, B, kappa, LdX<T>{tmp, g.ns}, active, EpiMgPost<T>{w, b, out, g.ns}, part, p, ks);
