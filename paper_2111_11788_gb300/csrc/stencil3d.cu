@@ -357,9 +357,9 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3(Grid g, const T* __restrict
 // the layer below plane p (S = PXY(p) + PXY(p - 1)), once per element, in
 // shared memory; a node takes the 2 x 2 sums of Q of the two layers around
 // it (B, one carried from the plane before) and its 6 face neighbours
-// weighted by the edge sums. About 19 FP64 operations per node instead of
+// weighted by the edge sums. About 17.5 FP64 operations per node instead of
 // the 33 of k_zm3 (the kernel is bound by the FP64 pipe; the 4 node arrays
-// of kappa sums, [K_n | K_x | K_y | K_z] per sample, are computed once per
+// of kappa sums, [5 K_n | K_x | K_y | K_z] per sample, are computed once per
 // solve by k_ksum3). Same tiles, chunks, loaders, epilogues and boundary
 // rule as k_zm3.
 template <class Ld, class Epi>
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3q(Grid g, const double* __re
   const double h12 = g.c12;   // h / 12
   // per output row: B of the layer below the current output plane, the
   // centre u and K_z of the plane below it, the kappa sums of the output
-  // plane (K_n, K_x(i), K_x(i - 1), K_y(j), K_y(j - 1), K_z) loaded a plane
+  // plane (5 K_n, K_x(i), K_x(i - 1), K_y(j), K_y(j - 1), K_z) loaded a plane
   // ahead, and the epilogue inputs
   double Bprev[ZRY], ucar[ZRY], kzcar[ZRY], ks[ZRY][6];
   typename Epi::Pre pre[ZRY];
@@ -493,15 +493,14 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3q(Grid g, const double* __re
         const bool in = cint[r] && m >= 1 && m < n;
         double acc = 0.0;
         if (in) {
-          // the six face neighbours by their edge sums, then 5 u K_n - sum kappa_e S_e
-          double sx = ks[r][1] * v[1];
+          // - sum kappa_e S_e, the six face neighbours by their edge sums, 5 u K_n
+          double sx = fma(ks[r][1], v[1], -(Bprev[r] + Bcur));
           sx = fma(ks[r][2], v[-1], sx);
           sx = fma(ks[r][3], v[ZSX], sx);
           sx = fma(ks[r][4], v[-ZSX], sx);
           sx = fma(ks[r][5], svb[vbase + r * ZSX], sx);
           sx = fma(kzcar[r], ucar[r], sx);
-          sx = fma(5.0 * uc, ks[r][0], sx);
-          acc = sx - (Bprev[r] + Bcur);
+          acc = fma(uc, ks[r][0], sx);
         }
         double done;
         if constexpr (Epi::kRes) done = fma(-h12, acc, epi.rhs(pre[r]));
@@ -526,7 +525,7 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3q(Grid g, const double* __re
   prof_tick3(prof);
 }
 
-// Kappa sums of every node (0 outside the mesh), per sample [K_n | K_x | K_y
+// Kappa sums of every node (0 outside the mesh), per sample [5 K_n | K_x | K_y
 // | K_z] in node strides: K_n the 8 elements around the node, K_x the 4
 // elements sharing the edge to the +x neighbour (element column i, rows j-1
 // and j, layers k-1 and k), K_y and K_z likewise. Once per solve.
@@ -557,7 +556,7 @@ __global__ void __launch_bounds__(256) k_ksum3(Grid g, const double* __restrict_
     double L1, X1, Y1;
     layer(kz, L1, X1, Y1);
     const int64_t o = ((int64_t)kz * N1 + c.j) * N1 + c.i;
-    kn[o] = L0 + L1;
+    kn[o] = 5.0 * (L0 + L1);
     kn[g.ns + o] = Y0 + Y1;
     kn[2 * g.ns + o] = X0 + X1;
     kn[3 * g.ns + o] = L1;
