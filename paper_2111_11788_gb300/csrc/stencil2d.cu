@@ -508,7 +508,9 @@ __global__ void __launch_bounds__(SBLOCK) k_pq2(Grid g, const T* __restrict__ K,
   prof_tick(prof);
 }
 
-// Pre-smoothing from zero and residual: e = W b, r1 = b - A e.
+// Pre-smoothing from zero and residual: e = W b, r1 = b - A e. In FP32 e is not
+// stored: the post-smoother, bound by issue and bytes, forms it again from the
+// W and b it reads anyway; in FP64, bound by the FP64 pipe, it is.
 template <class T, bool C, int SR>
 __global__ void __launch_bounds__(SBLOCK) k_mgpre2(Grid g, const T* __restrict__ K, int64_t cs,
                                                    const T* __restrict__ W,
@@ -541,9 +543,8 @@ __global__ void __launch_bounds__(SBLOCK) k_mgpre2(Grid g, const T* __restrict__
                            return Pair<T>{__ldg(w_ + o), __ldg(bv + o)};
                          },
                          [&](const Pair<T>& r, int, int) { return r.a * r.b; },
-                         [&](int j, T ev, T ax) {
+                         [&](int j, T, T ax) {
                            const int64_t o = (int64_t)j * s.N1 + s.c;
-                           e[o] = ev;
                            r1[o] = interior2(s.n, s.c, j) ? __ldg(bv + o) - ax : T(0);
                          });
   }
@@ -692,7 +693,6 @@ template <int SR>
 __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, const float* __restrict__ K,
                                                         const float* __restrict__ W,
                                                         const float* __restrict__ Bv,
-                                                        const float* __restrict__ E,
                                                         const float* __restrict__ Ec, float* __restrict__ Out,
                                                         const int32_t* __restrict__ active,
                                                         double* __restrict__ part, Prof prof) {
@@ -701,7 +701,6 @@ __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, con
   const Strip s = strip_of<SR>(g);
   const int nc = g.n / 2;
   const float* ec = Ec + b * nsc;
-  const float* e = E + b * g.ns;
   const float* w_ = W + b * g.ns;
   const float* bv = Bv + b * g.ns;
   float* out = Out + b * g.ns;
@@ -732,37 +731,39 @@ __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, con
     hrow(s.y0 / 2 - 1, a, bb);
     hprev = a + bb;
   }
-  // The pair of field rows (j, j + 1) is formed in the step that outputs rows
-  // j - 1 and j, so its fetch also loads b and W of those two rows (bw):
-  // they get the same step of latency as the field.
+  // e = W b is formed from the rows' W and b (bitwise the product a separate
+  // pass would store). The pair of field rows (j, j + 1) is formed in the step
+  // that outputs rows j - 1 and j, whose own b and W are those of the pair
+  // before (row j - 1, carried) and of this one (row j).
   struct RawPE {
-    float e0, e1, a, b, b0, b1, w0, w1;
+    float b0, w0, b1, w1, a, b;
   };
   float bw[4] = {0.f, 0.f, 0.f, 0.f};   // b, W of the even and the odd output row of the step
+  float bn = 0.f, wn = 0.f;             // b, W of the pair's second row, the next step's even output row
   stream_strip_pair(
       s, K + b * g.es,
       [&](int j) {
         RawPE r;
-        const float* ej = e + (j * s.N1 + c);
-        r.e0 = interior2(n, c, j) ? __ldg(ej) : 0.f;
-        r.e1 = interior2(n, c, j + 1) ? __ldg(ej + s.N1) : 0.f;
+        const int o = j * s.N1 + c;
+        const bool in0 = interior2(n, c, j), in1 = interior2(n, c, j + 1);
+        r.b0 = in0 ? __ldg(bv + o) : 0.f;
+        r.w0 = in0 ? __ldg(w_ + o) : 0.f;
+        r.b1 = in1 ? __ldg(bv + o + s.N1) : 0.f;
+        r.w1 = in1 ? __ldg(w_ + o + s.N1) : 0.f;
         hrow((j + 1) >> 1, r.a, r.b);
-        const bool o0 = s.out && interior2(n, c, j - 1), o1 = s.out && interior2(n, c, j);
-        r.b0 = o0 ? __ldg(bv + (j - 1) * s.N1 + c) : 0.f;
-        r.w0 = o0 ? __ldg(w_ + (j - 1) * s.N1 + c) : 0.f;
-        r.b1 = o1 ? __ldg(bv + j * s.N1 + c) : 0.f;
-        r.w1 = o1 ? __ldg(w_ + j * s.N1 + c) : 0.f;
         return r;
       },
       [&](const RawPE& r, int j) {
         const float h = r.a + r.b;
-        const float x0 = interior2(n, c, j) ? fmaf(0.25f, hprev + h, r.e0) : 0.f;
-        const float x1 = interior2(n, c, j + 1) ? fmaf(0.5f, h, r.e1) : 0.f;
+        const float x0 = interior2(n, c, j) ? fmaf(0.25f, hprev + h, __fmul_rn(r.w0, r.b0)) : 0.f;
+        const float x1 = interior2(n, c, j + 1) ? fmaf(0.5f, h, __fmul_rn(r.w1, r.b1)) : 0.f;
         hprev = h;
-        bw[0] = r.b0;
-        bw[1] = r.w0;
-        bw[2] = r.b1;
-        bw[3] = r.w1;
+        bw[0] = bn;
+        bw[1] = wn;
+        bw[2] = r.b0;
+        bw[3] = r.w0;
+        bn = r.b1;
+        wn = r.w1;
         return make_float2(x0, x1);
       },
       [&](int j, float ev, float ax) {
@@ -1599,7 +1600,7 @@ cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* 
       k_mgpost2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, coef, coef_stride(g), w, b, e, ec, out,
                                                         active, part, p);
     else if constexpr (sizeof(T) == 4)
-      k_mgpost2f<SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, w, b, e, ec, out, active, part, p);
+      k_mgpost2f<SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, w, b, ec, out, active, part, p);
     else
       k_mgpost2<T, false, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, g.es, w, b, e, ec, out,
                                                          active, part, p);
