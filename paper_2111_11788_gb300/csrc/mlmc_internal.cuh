@@ -51,6 +51,7 @@ enum KernelId {
   KID_REFINE,
   KID_RESID64,
   KID_MG_BOTTOM,
+  KID_RESIDENT,
   NUM_KERNELS
 };
 
@@ -384,6 +385,43 @@ inline cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coar
                     : d3::prolong_guess(s, g, coarse, uc, x, active, B, p);
 }
 }  // namespace op
+
+// Whole solves of a batch on a small mesh (resident.cu): FP64 (T double) or
+// the mixed form (T float). Arrays as in the separate kernels' workspace.
+constexpr int MAX_RESIDENT_LEVELS = 7;
+template <class T>
+struct ResidentSolve {
+  int K;                              // multigrid levels (1: Jacobi)
+  Grid g[MAX_RESIDENT_LEVELS];
+  T* kap[MAX_RESIDENT_LEVELS];        // [0]: FP64 form given; mixed form made from kap64 (round_kappa) or given
+  T* coef[MAX_RESIDENT_LEVELS];       // FP64 2D coefficient blocks, else null
+  T* w[MAX_RESIDENT_LEVELS];
+  double omega;
+  bool round_kappa;
+  const double* kap64;                // mixed form: the FP64 kappa and (2D) its coefficient block
+  double* coef64;
+  double tol;                         // stop at ||r|| <= tol
+  int max_iter;                       // CG cap (mixed form: of each inner solve)
+  double inner_rtol, scale0;
+  int outer_max;
+  const double* uc;                   // nested guess on the next coarser mesh (node stride ucs), or null
+  int64_t ucs;
+  double* u;
+  double* q;
+  int32_t *iters, *iters2;            // iters2 may be null
+  int box, L, H;
+  double inv_vol;
+};
+// CTAs a resident solve may take in a round that also solves larger meshes: it
+// holds all its CTAs' registers while it waits on barriers, and the larger
+// meshes' kernels, which fill the HBM or the FP64 pipe, run beside it (a mixed
+// 2D run of 32^2 .. 512^2: 21.1 ms with no limit, 20.5 with 304 CTAs, 19.9 with
+// 152, 19.7 with 114, 20.4 with 76, 25.9 with 38).
+constexpr int64_t RESIDENT_SHARED_CTAS = 114;
+// 0 where the resident solve does not run (a function of mesh and form alone)
+int resident_bands(int dim, int n, int K, bool mixed);
+template <class T>
+cudaError_t launch_resident(cudaStream_t s, const ResidentSolve<T>& r, int64_t B, int64_t slots, int* launches);
 
 cudaError_t launch_finalize(cudaStream_t s, FinMode mode, const double* part, int64_t tiles,
                             const Scalars& sc, double* out, int iter, int max_iter, int64_t B,

@@ -58,7 +58,7 @@ namespace {
 const char* kKernelNames[NUM_KERNELS] = {
     "draw_xi", "kle_table", "kappa", "coarsen_kappa", "apply", "pcg_init", "pcg_pq", "pcg_xr",
     "jacobi_z", "mg_pre", "restrict", "coarse_solve", "mg_post", "qoi", "finalize", "welford",
-    "estimate", "count_active", "setup", "refine", "resid64", "mg_bottom"};
+    "estimate", "count_active", "setup", "refine", "resid64", "mg_bottom", "resident"};
 
 // Bump allocator over the workspace (base == nullptr: size only).
 struct Carve {
@@ -291,6 +291,7 @@ struct mlmc_plan_s {
   double ms[NUM_KERNELS] = {0};
   int64_t kl[NUM_KERNELS] = {0};
   int64_t launches = 0;
+  int64_t resident_slots = 0;   // CTAs that resident solves of the round being captured may take (0: any number)
   bool zw_used = false;   // mlmc_apply32 ran the 3D FP32 z-march (bounded waits to check)
   // graph-captured solves, keyed by (form, mesh, batch, workspace) and the
   // arrays they bake in (kappa, solution, QoI, iteration counts, guess)
@@ -1078,10 +1079,79 @@ mlmc_status fp64_epilogue(mlmc_plan p, const MeshInfo& mi, SolveWs<double>& w, i
   return MLMC_OK;
 }
 
+// Whether the solves on this mesh run as one resident launch (resident.cu).
+bool resident(const MeshInfo& mi, bool mixed) {
+  return mi.K <= MAX_RESIDENT_LEVELS && resident_bands(mi.g[0].dim, mi.n, mi.K, mixed) > 0;
+}
+
+template <class T>
+ResidentSolve<T> resident_args(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, double* q_dev, int32_t* iters_dev,
+                               const Guess& gs) {
+  const mlmc_config& c = p->cfg;
+  ResidentSolve<T> r{};
+  r.K = mi.K;
+  for (int k = 0; k < mi.K; ++k) {
+    r.g[k] = mi.g[k];
+    r.kap[k] = w.kap[k];
+    r.coef[k] = mi.g[0].dim == 2 ? w.coef[k] : nullptr;
+    r.w[k] = w.w[k];
+  }
+  r.omega = mi.K > 1 ? c.mg_omega : 1.0;
+  r.tol = c.rtol * b_norm(c, mi.g[0]);
+  r.uc = gs.uc;
+  r.ucs = gs.gc.ns;
+  r.q = q_dev;
+  r.iters2 = iters_dev;
+  r.box = (c.qoi == MLMC_QOI_BOX_MEAN) ? 1 : 0;
+  r.L = (int)std::lround(c.box_lo * mi.n);
+  r.H = (int)std::lround(c.box_hi * mi.n);
+  r.inv_vol = r.box ? 1.0 / std::pow(c.box_hi - c.box_lo, c.dim) : 1.0;
+  return r;
+}
+
+template <class T>
+mlmc_status run_resident(mlmc_plan p, const ResidentSolve<T>& r, int64_t B) {
+  int launches = 1;
+  CK(run(p, KID_RESIDENT, [&] { return launch_resident<T>(p->stream, r, B, p->resident_slots, &launches); }));
+  p->launches += launches - 1;
+  return MLMC_OK;
+}
+
+mlmc_status resident_fp64(mlmc_plan p, const MeshInfo& mi, SolveWs<double>& w, int64_t B, double* q_dev,
+                          int32_t* iters_dev, const Guess& gs) {
+  ResidentSolve<double> r = resident_args<double>(p, mi, w, q_dev, iters_dev, gs);
+  r.max_iter = p->cfg.max_iter;
+  r.u = w.x;
+  r.iters = w.sc.iters;
+  return run_resident(p, r, B);
+}
+
+mlmc_status resident_mixed(mlmc_plan p, const MeshInfo& mi, MixedWs& w, int64_t B, double* q_dev,
+                           int32_t* iters_dev, const Guess& gs) {
+  const mlmc_config& c = p->cfg;
+  ResidentSolve<float> r = resident_args<float>(p, mi, w.in, q_dev, iters_dev, gs);
+  r.round_kappa = !(w.xi32 && c.kle_tensor);
+  if (!r.round_kappa)
+    CK(run(p, KID_KAPPA, [&] {
+      return launch_kappa32(p->stream, mi.g[0], c.modes_per_dim, p->sqrt_sigma2, mi.table, w.xi32, p->M,
+                               p->d_slot, B, w.in.kap[0]);
+    }));
+  r.kap64 = w.kap64;
+  r.coef64 = mi.g[0].dim == 2 ? w.coef64 : nullptr;
+  r.max_iter = c.inner_max_iter;
+  r.inner_rtol = c.inner_rtol;
+  r.outer_max = c.outer_max_iter;
+  r.scale0 = b_norm(c, mi.g[0]);
+  r.u = w.u;
+  r.iters = w.outer.iters;
+  return run_resident(p, r, B);
+}
+
 // FP64 solve issued into the graph being captured: setup -> while(two PCG
 // iterations + loop control) -> QoI epilogue.
 mlmc_status issue_fp64(mlmc_plan p, const MeshInfo& mi, SolveWs<double>& w, int64_t B,
                        double* q_dev, int32_t* iters_dev, const Guess& gs) {
+  if (resident(mi, false)) return resident_fp64(p, mi, w, B, q_dev, iters_dev, gs);
   mlmc_status st = fp64_setup(p, mi, w, B, gs);
   if (st != MLMC_OK) return st;
   const MeshInfo* mip = &mi;
@@ -1100,6 +1170,7 @@ mlmc_status issue_fp64(mlmc_plan p, const MeshInfo& mi, SolveWs<double>& w, int6
 mlmc_status solve_fp64(mlmc_plan p, int mesh, const MeshInfo& mi, SolveWs<double>& w, int64_t B,
                        double* q_dev, int32_t* iters_dev, const Guess& gs) {
   const mlmc_config& c = p->cfg;
+  if (resident(mi, false)) return resident_fp64(p, mi, w, B, q_dev, iters_dev, gs);
   if (!graphs_on(p)) {
     mlmc_status st = fp64_setup(p, mi, w, B, gs);
     if (st != MLMC_OK) return st;
@@ -1213,6 +1284,7 @@ mlmc_status mixed_epilogue(mlmc_plan p, const MeshInfo& mi, MixedWs& w, int64_t 
 // while_outer(pre, re-arm inner, while_inner(PCG), post, outer control) -> QoI.
 mlmc_status issue_mixed(mlmc_plan p, const MeshInfo& mi, MixedWs& w, int64_t B, double* q_dev,
                         int32_t* iters_dev, const Guess& gs) {
+  if (resident(mi, true)) return resident_mixed(p, mi, w, B, q_dev, iters_dev, gs);
   mlmc_status st = mixed_setup(p, mi, w, B, gs);
   if (st != MLMC_OK) return st;
   const MeshInfo* mip = &mi;
@@ -1250,6 +1322,7 @@ mlmc_status solve_mixed(mlmc_plan p, int mesh, const MeshInfo& mi, MixedWs& w, i
                         double* q_dev, int32_t* iters_dev, const Guess& gs) {
   cudaStream_t s = p->stream;
   const mlmc_config& c = p->cfg;
+  if (resident(mi, true)) return resident_mixed(p, mi, w, B, q_dev, iters_dev, gs);
   if (!graphs_on(p)) {
     mlmc_status st = mixed_setup(p, mi, w, B, gs);
     if (st != MLMC_OK) return st;
@@ -1419,6 +1492,8 @@ mlmc_status round_launch(mlmc_plan p, const std::vector<int64_t>& first,
     st = build_graph(p, [&]() -> mlmc_status {
       cudaStream_t origin = p->stream;
       const size_t nc = chunks.size();
+      for (const auto& ch : chunks)
+        if (!resident(p->meshes[ch.level], mixed)) p->resident_slots = RESIDENT_SHARED_CTAS;
       cudaEvent_t fork = p->branch_ev[0];
       CK(cudaEventRecord(fork, origin));
       // chunks finest level first, each on its own branch
@@ -1436,6 +1511,7 @@ mlmc_status round_launch(mlmc_plan p, const std::vector<int64_t>& first,
         p->stream = origin;
         if (s2 == MLMC_OK) CK(cudaEventRecord(p->branch_ev[1 + order[i]], S));
       }
+      p->resident_slots = 0;
       // each level's chunks are folded in sample order on the branch of its first chunk
       for (int l = 0; l < L1 && s2 == MLMC_OK; ++l) {
         int head = -1;
@@ -1579,6 +1655,8 @@ mlmc_status group_launch(mlmc_plan p, const std::vector<int64_t>& first, char* w
     CK(cudaEventRecord(p->branch_ev[0], origin));
     int nb = 0;
     mlmc_status s2 = MLMC_OK;
+    for (int l = 0; l < L1; ++l)
+      if (B[l] > 0 && !resident(p->meshes[l], mixed)) p->resident_slots = RESIDENT_SHARED_CTAS;
     for (int l = L1 - 1; l >= 0 && s2 == MLMC_OK; --l) {
       if (B[l] <= 0) continue;
       cudaStream_t S = p->branch[nb];
@@ -1589,6 +1667,7 @@ mlmc_status group_launch(mlmc_plan p, const std::vector<int64_t>& first, char* w
       if (s2 == MLMC_OK) CK(cudaEventRecord(p->branch_ev[1 + nb], S));
       ++nb;
     }
+    p->resident_slots = 0;
     for (int i = 0; i < nb && s2 == MLMC_OK; ++i) CK(cudaStreamWaitEvent(origin, p->branch_ev[1 + i], 0));
     return s2;
   }, &rec);
