@@ -108,8 +108,8 @@ inline cudaError_t once_per_device(std::atomic<uint64_t>& done, F&& set) {
   return e;
 }
 
-// The small multigrid levels k0 .. K-1 of a V-cycle fused into one kernel,
-// one CTA per sample in shared memory: from b at level k0 (restricted by the
+// The small multigrid levels k0 .. K-1 of a V-cycle fused into one kernel, a
+// cluster of CTAs per sample in shared memory: from b at level k0 (restricted by the
 // level above) to the post-smoothed correction out at level k0. Per level:
 // the grid, kappa, W and (2D FP64: non-null) operator coefficients; sample
 // strides as in the unfused kernels.
@@ -240,9 +240,6 @@ cudaError_t add_correction(cudaStream_t s, const Grid& g, double* u, const float
 cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, const double* uc,
                           double* x, const int32_t* active, int64_t B, Prof p);
 
-template <class T>
-cudaError_t mg_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b, T* out,
-                      const int32_t* active, int64_t B, Prof p);
 }  // namespace d2
 
 // iter_dev (may be null) overrides iter with a device-side iteration counter.
@@ -288,9 +285,6 @@ cudaError_t ksum(cudaStream_t s, const Grid& g, const double* kappa, double* ks,
 // nested initial guess: x = P uc (trilinear interpolation from grid `coarse`)
 cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, const double* uc,
                           double* x, const int32_t* active, int64_t B, Prof p);
-template <class T>
-cudaError_t mg_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b, T* out,
-                      const int32_t* active, int64_t B, Prof p);
 // bounded waits of the FP32 z-march that gave up (a copy never landed) since
 // the last call on this device; resets the count
 cudaError_t take_wait_timeouts(cudaStream_t s, unsigned* out);
@@ -373,12 +367,6 @@ inline cudaError_t add_correction(cudaStream_t s, const Grid& g, double* u, cons
                                   const double* scale, const int32_t* active, int64_t B, Prof p) {
   return d2::add_correction(s, g, u, d32, scale, active, B, p);
 }
-template <class T>
-inline cudaError_t mg_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b, T* out,
-                             const int32_t* active, int64_t B, Prof p) {
-  return lv.g[0].dim == 2 ? d2::mg_bottom<T>(s, lv, b, out, active, B, p)
-                          : d3::mg_bottom<T>(s, lv, b, out, active, B, p);
-}
 inline cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, const double* uc,
                                  double* x, const int32_t* active, int64_t B, Prof p) {
   return g.dim == 2 ? d2::prolong_guess(s, g, coarse, uc, x, active, B, p)
@@ -422,6 +410,10 @@ constexpr int64_t RESIDENT_SHARED_CTAS = 114;
 int resident_bands(int dim, int n, int K, bool mixed);
 template <class T>
 cudaError_t launch_resident(cudaStream_t s, const ResidentSolve<T>& r, int64_t B, int64_t slots, int* launches);
+// The fused small levels of a V-cycle (resident.cu).
+template <class T>
+cudaError_t launch_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b, T* out, const int32_t* active,
+                          int64_t B, Prof p);
 
 cudaError_t launch_finalize(cudaStream_t s, FinMode mode, const double* part, int64_t tiles,
                             const Scalars& sc, double* out, int iter, int max_iter, int64_t B,

@@ -724,7 +724,7 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
       bytes += nodes_of(mi.g[k0 + l]) + elems_of(mi.g[k0 + l]);
     }
     CK(run(p, KID_MG_BOTTOM, [&] {
-      return op::mg_bottom<T>(s, lv, w.bk[k0], w.eo[k0], w.sc.active, B,
+      return launch_bottom<T>(s, lv, w.bk[k0], w.eo[k0], w.sc.active, B,
                               prof_for(p, KID_MG_BOTTOM, bytes * vb));
     }));
   } else {

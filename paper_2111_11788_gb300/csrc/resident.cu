@@ -359,7 +359,8 @@ struct Res {
     }
   }
   // z = M r (r: level 0's b, with e = W r in place; z: its output array); hands
-  // in the parts of r.z
+  // in the parts of r.z (Dot)
+  template <bool Dot>
   __device__ __forceinline__ void vcycle() const {
     T dot = T(0);
     for (int l = 0; l < a.K - 1; ++l) {
@@ -393,9 +394,9 @@ struct Res {
         stencil(l, L.oe, [&](int x) { return b[x]; }, [&](int x, int g, T r) {
           const T v = fma(__ldg(w + g), r, e[x]);
           t[x] = v;
-          if (l == 0) dot = fma(b[x], v, dot);
+          if (Dot && l == 0) dot = fma(b[x], v, dot);
         }, [&](int v) {
-          part(0, v, dot);
+          if constexpr (Dot) part(0, v, dot);
           dot = T(0);
         });
       }
@@ -423,7 +424,7 @@ struct Res {
     if (mg) {
       nodes(0, [&](int js, int o, int, int) { q[js * S + o] = __ldg(w + (z0 + js) * S + o) * r[js * S + o]; });
       all_sync();
-      vcycle();
+      vcycle<true>();
     } else nodes0([&](int js, int o, int, int) {
       const T rv = r[js * S + o];
       dot = fma(rv, __ldg(w + (z0 + js) * S + o) * rv, dot);
@@ -470,7 +471,7 @@ struct Res {
       });
       if (sc.stop) return sc.stop == 1 ? it : -1;
       if (mg) {
-        vcycle();
+        vcycle<true>();
         total<T>(1, [&](double rz, double) {
           sc.beta = sc.gamma != 0.0 ? rz / sc.gamma : 0.0;
           sc.gamma = rz;
@@ -638,6 +639,58 @@ __global__ void __launch_bounds__(RES_THREADS, RES_PER_SM) k_resident(const __gr
   }
 }
 
+// The levels of at most 64^2 (2D) or 16^3 (3D) cells below the finest of a
+// larger mesh's V-cycle, for a PCG of separate kernels: from b on the finest of
+// them to the post-smoothed correction out, with the same vcycle(). `cycles` 2:
+// a second cycle on the residual of the first.
+template <int DIM, class T>
+__global__ void __launch_bounds__(RES_THREADS, RES_PER_SM) k_bottom(const __grid_constant__ ResArgs<T> a,
+                                                                    const T* __restrict__ Bv, T* __restrict__ Out,
+                                                                    const int32_t* __restrict__ active, int cycles,
+                                                                    Prof prof) {
+  extern __shared__ __align__(16) unsigned char res_sm[];
+  const int tid = threadIdx.x;
+  Res<DIM, T, false> s{a, res_sm, (int)(blockIdx.x % a.C), (int64_t)(blockIdx.x / a.C), tid, 0};
+  if (!active[s.smp]) return;   // the whole cluster
+  for (unsigned k = tid; k < a.bytes / 8; k += RES_THREADS) reinterpret_cast<double*>(res_sm)[k] = 0.0;
+  __syncthreads();
+  const ResLevel<T>& L = a.lv[0];
+  const int S = L.S, z0 = s.first(0), cnt = s.own(0);
+  T* b = s.template at<T>(L.ob);
+  T* e = s.template at<T>(L.oe);
+  const T* t = s.template at<T>(L.ot);
+  const T* w = L.w + s.smp * L.ns;
+  const T* src = Bv + s.smp * L.ns;
+  T* out = Out + s.smp * L.ns;
+  s.nodes(0, [&](int js, int o, int, int) {
+    const int g = (z0 + js) * S + o;
+    const T v = src[g];
+    b[js * S + o] = v;
+    e[js * S + o] = __ldg(w + g) * v;
+  });
+  s.all_sync();   // the cluster has started and every array is in place
+  s.template vcycle<false>();
+  if (cycles > 1) {
+    s.all_sync();
+    for (int k = tid; k < cnt * S; k += RES_THREADS) out[z0 * S + k] = t[k];
+    s.stencil(0, L.ot, [&](int x) { return b[x]; },
+              [&](int x, int g, T r) {
+                b[x] = r;
+                e[x] = __ldg(w + g) * r;
+              }, [](int) {});
+    s.all_sync();
+    s.template vcycle<false>();
+  }
+  __syncthreads();
+  for (int k = tid; k < cnt * S; k += RES_THREADS) out[z0 * S + k] = cycles > 1 ? out[z0 * S + k] + t[k] : t[k];
+  if (s.rank == 0)
+    for (int k = tid; k < S; k += RES_THREADS) out[k] = T(0);
+  if (cnt > 0 && z0 + cnt == L.n)
+    for (int k = tid; k < S; k += RES_THREADS) out[L.n * S + k] = T(0);
+  if (prof.acc && s.rank == 0 && tid == 0) atomicAdd(prof.acc, prof.per_sample);
+  s.all_sync();   // no CTA leaves while another may read its arrays
+}
+
 // Setup, first launch: one CTA per sample makes the kappa hierarchy (mixed
 // form: the FP32 kappa of the finest mesh too, unless it is given).
 template <class T>
@@ -738,7 +791,7 @@ __global__ void __launch_bounds__(256) k_res_coefs(const __grid_constant__ ResCo
 // Fills the geometry and the shared-memory layout of `a` for C CTAs per
 // sample; returns the dynamic shared memory of a CTA.
 template <class T>
-static size_t resident_layout(int dim, int n, int K, int V, int C, ResArgs<T>& a) {
+static size_t resident_layout(int dim, int n, int K, int V, int C, ResArgs<T>& a, bool solve = true) {
   unsigned off = 0;
   auto take = [&](int64_t count, size_t size) {
     off = (off + 15u) / 16u * 16u;
@@ -778,12 +831,14 @@ static size_t resident_layout(int dim, int n, int K, int V, int C, ResArgs<T>& a
     L.oe = last ? 0 : take(band, sizeof(T));
     L.ot = K > 1 ? take(band, sizeof(T)) : 0;
   }
-  a.ox = take(band0, sizeof(T));
-  a.op = take(band0, sizeof(T));
   a.oz = take(a.lv[0].S, sizeof(T));
-  a.ored = take(4 * 2 * RES_MAX_V, 8);
-  a.osw = take((int64_t)(K > 1 ? 1 : 2) * a.nv * RES_THREADS, 8);
-  a.osc = take(1, sizeof(ResScalars));
+  if (solve) {
+    a.ox = take(band0, sizeof(T));
+    a.op = take(band0, sizeof(T));
+    a.ored = take(4 * 2 * RES_MAX_V, 8);
+    a.osw = take((int64_t)(K > 1 ? 1 : 2) * a.nv * RES_THREADS, 8);
+    a.osc = take(1, sizeof(ResScalars));
+  }
   a.bytes = (off + 15u) / 16u * 16u;
   return a.bytes;
 }
@@ -928,4 +983,55 @@ cudaError_t launch_resident(cudaStream_t s, const ResidentSolve<T>& r, int64_t B
 template cudaError_t launch_resident<double>(cudaStream_t, const ResidentSolve<double>&, int64_t, int64_t, int*);
 template cudaError_t launch_resident<float>(cudaStream_t, const ResidentSolve<float>&, int64_t, int64_t, int*);
 
+template <int DIM, class T>
+static cudaError_t launch_bottom_dim(cudaStream_t s, const ResArgs<T>& a, const T* b, T* out, const int32_t* active,
+                                     int cycles, int64_t B, Prof p) {
+  static std::atomic<uint64_t> opted{0};
+  cudaError_t e = once_per_device(opted, [] {
+    return cudaFuncSetAttribute(k_bottom<DIM, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RES_SMEM_MAX);
+  });
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(B * a.C), 1, 1);
+  cfg.blockDim = dim3(RES_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = a.bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)a.C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, k_bottom<DIM, T>, a, b, out, active, cycles, p);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b, T* out, const int32_t* active,
+                          int64_t B, Prof p) {
+  const int dim = lv.g[0].dim, n = lv.g[0].n;
+  if (lv.L < 2 || lv.L > RES_MAX_LEVELS || lv.g[lv.L - 1].n != 2) return cudaErrorInvalidValue;
+  // as many CTAs per sample as the batch leaves room for (nothing is summed
+  // over a sample here, so the result does not depend on it), at least as
+  // many as its arrays need
+  int C = 1;
+  while (C < RES_MAX_V && ipow(n - 1, dim) > (int64_t)C * RES_THREADS && 2 * C <= n) C *= 2;
+  ResArgs<T> a{};
+  while (C > 1 && B * C > RES_SLOTS && resident_layout(dim, n, lv.L, C / 2, C / 2, a, false) <= RES_SMEM_SHARE) C /= 2;
+  if (resident_layout(dim, n, lv.L, C, C, a, false) > RES_SMEM_MAX) return cudaErrorInvalidValue;
+  for (int l = 0; l < lv.L; ++l) {
+    a.lv[l].ns = lv.g[l].ns;
+    a.lv[l].es = lv.g[l].es;
+    a.lv[l].kap = lv.kap[l];
+    a.lv[l].coef = lv.coef[l];
+    a.lv[l].w = lv.w[l];
+  }
+  return dim == 2 ? launch_bottom_dim<2, T>(s, a, b, out, active, lv.cycles, B, p)
+                  : launch_bottom_dim<3, T>(s, a, b, out, active, lv.cycles, B, p);
+}
+template cudaError_t launch_bottom<double>(cudaStream_t, const BottomLevels<double>&, const double*, double*,
+                                           const int32_t*, int64_t, Prof);
+template cudaError_t launch_bottom<float>(cudaStream_t, const BottomLevels<float>&, const float*, float*,
+                                          const int32_t*, int64_t, Prof);
 }  // namespace mlmc

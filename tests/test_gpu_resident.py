@@ -117,3 +117,16 @@ def test_a_round_with_larger_meshes(m, precision):
             y = np.asarray(qf) - (np.asarray(qc) if level else 0.0)
             # Welford's update rounds a few ulps of the largest value per sample
             assert n == count and abs(mean - y.mean()) <= 4 * count * 2.0 ** -53 * np.abs(y).max()
+
+
+@pytest.mark.parametrize("dim,n,precision,count", [(2, 256, "fp64", 120), (2, 256, "mixed", 120), (2, 512, "mixed", 60),
+                                                   (3, 32, "fp64", 240), (3, 64, "mixed", 120)])
+def test_fused_levels_do_not_depend_on_the_batch(m, dim, n, precision, count):
+    """Larger meshes: the V-cycle's small levels on a cluster whose size follows the batch."""
+    kap = random_element_field(dim, n, 2, seed=6, spread=0.5)
+    _, u, q, it = solve(m, dim, n, "gmg", precision, np.concatenate([kap] * (count // 2)))
+    assert np.all(it > 0)
+    for s in (0, 1):
+        _, u1, q1, it1 = solve(m, dim, n, "gmg", precision, kap[s:s + 1])
+        for k in (s, count - 2 + s):
+            assert np.array_equal(u1[0], u[k]) and q1[0] == q[k] and it1[0] == it[k]

@@ -9,7 +9,7 @@ import pytest
 THREADS, BAND, MAX_V, MAX_LEVELS, SMEM, SHARE = 256, 512, 8, 7, 224 * 1024, 74 * 1024
 
 
-def layout(dim, n, K, V, C, mixed):
+def layout(dim, n, K, V, C, mixed, solve=True):
     """(levels, nd, bytes): the geometry and shared memory of one CTA."""
     size = 4 if mixed else 8
     off = 0
@@ -32,12 +32,13 @@ def layout(dim, n, K, V, C, mixed):
         lv.append(dict(n=nl, N1=N1, S=S, R=R, m1=-(-2 ** 32 // m) % 2 ** 32, m2=-(-2 ** 32 // (m * m)) % 2 ** 32))
         for _ in range((0 if K > 1 and l == K - 1 else 2) + (1 if K > 1 else 0)):
             take(R * S, size)
-    for _ in range(2):
-        take(lv[0]["R"] * lv[0]["S"], size)
     take(lv[0]["S"], size)
-    take(4 * 2 * MAX_V, 8)
-    take((1 if K > 1 else 2) * nv * THREADS, 8)
-    take(48, 1)
+    if solve:
+        for _ in range(2):
+            take(lv[0]["R"] * lv[0]["S"], size)
+        take(4 * 2 * MAX_V, 8)
+        take((1 if K > 1 else 2) * nv * THREADS, 8)
+        take(48, 1)
     lv[0]["rv"] = rv
     return lv, nd, (off + 15) // 16 * 16
 
@@ -131,3 +132,23 @@ def check(dim, n, K, mixed, V, C):
                 assert all(slab(f) is not None for f in (2 * z - 1, 2 * z, 2 * z + 1)) and 2 * (nc - 1) + 1 <= nl
             for z in range(1, nl):       # prolongation reads coarse slabs z / 2 (and z / 2 + 1 for odd z)
                 assert 0 <= z >> 1 and (z >> 1) + (z & 1) <= nc and ((nl - 1) >> 1) + 1 <= nc
+
+
+BOTTOM_SLOTS = 152 * 3
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("dim,n,K", [(2, 1 << k, k) for k in range(2, 7)] + [(3, 1 << k, k) for k in range(2, 5)])
+def test_bottom_levels_fit_every_batch(dim, n, K, mixed):
+    """The V-cycle's fused levels: the CTAs a batch gives a sample, each with room for its arrays."""
+    top = 1
+    while top < MAX_V and (n - 1) ** dim > top * THREADS and 2 * top <= n:
+        top *= 2
+    for B in (1, 40, 57, 58, 100, 500, 60000):
+        C = top
+        while C > 1 and B * C > BOTTOM_SLOTS and layout(dim, n, K, C // 2, C // 2, mixed, False)[2] <= SHARE:
+            C //= 2
+        lv, nd, bytes_ = layout(dim, n, K, C, C, mixed, False)
+        assert bytes_ <= SMEM and nd <= K - 1 and (C == 1) == (nd == 0)
+        for l in range(nd):
+            assert lv[l]["R"] * C == lv[l]["n"]
