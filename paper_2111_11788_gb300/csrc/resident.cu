@@ -421,6 +421,9 @@ struct Res {
       part(0, v, dot);
       dot = T(0);
     };
+    // what follows deals the nodes to the threads band by band, or all bands at
+    // once, unlike the caller that wrote r
+    __syncthreads();
     if (mg) {
       nodes(0, [&](int js, int o, int, int) { q[js * S + o] = __ldg(w + (z0 + js) * S + o) * r[js * S + o]; });
       all_sync();

@@ -130,3 +130,16 @@ def test_fused_levels_do_not_depend_on_the_batch(m, dim, n, precision, count):
         _, u1, q1, it1 = solve(m, dim, n, "gmg", precision, kap[s:s + 1])
         for k in (s, count - 2 + s):
             assert np.array_equal(u1[0], u[k]) and q1[0] == q[k] and it1[0] == it[k]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("dim,solver,n0,count", [(2, "gmg", 32, 130), (2, "jacobi", 22, 150), (3, "gmg", 8, 150)])
+def test_coupled_batches_repeat_bitwise(m, dim, solver, n0, count, precision):
+    """CTAs of several bands: a batch gives the same bits every time, and each sample the bits of a call of its own."""
+    wl = small_case(dim, n0=n0, levels=2, m=3, solver=solver, precision=precision)
+    with m.Plan(m.config_from_workload(wl), stream()) as plan:
+        one = [plan.sample_level(1, k, 1) for k in range(count)]
+        want = [np.concatenate([np.atleast_1d(o[i]) for o in one]) for i in (0, 1)]
+        for _ in range(8):
+            qf, qc, _ = plan.sample_level(1, 0, count)
+            assert np.array_equal(qf, want[0]) and np.array_equal(qc, want[1])
