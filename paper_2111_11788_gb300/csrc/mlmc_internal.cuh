@@ -80,6 +80,7 @@ struct Grid {
   int sx, sy;       // 2D: stencil CTAs per sample (strip groups x row chunks);
                     // 3D: node-tile CTAs per sample of the pointwise kernels (sx)
   int zc;           // 3D: z-planes per CTA of the z-marching stencil kernels
+  bool zset;        // 3D: zc is the caller's choice
   int zt;           // 3D FP32 z-march tiles: 0 = full width by TMA where possible, 1 = 32 x 16
   int zx;           // 3D: z-marching CTAs per sample
   int64_t tiles_s;  // partials per sample written by stencil kernels

@@ -43,6 +43,7 @@ Grid make_grid(int dim, int n, int z_chunk, int stencil_tile) {
     g.sy = 1;
     g.zc = (n + 1 <= 24) ? n + 1 : 16;
     if (z_chunk > 0) g.zc = std::min(z_chunk, n + 1);
+    g.zset = z_chunk > 0;
     g.zx = ((n + 31) / 32) * ((n + 15) / 16) * ((n + 1 + g.zc - 1) / g.zc);
     g.tiles_s = g.zx;
   }

@@ -1695,6 +1695,36 @@ inline bool zm_wide(const Grid& g) {
          (g.zx == (int64_t)(g.n / zw_rows(g.n, 2)) * ((g.n + 1 + g.zc - 1) / g.zc));
 }
 
+// The grid with the z-chunks of a launch that leaves no partial sums (A x, the
+// pre-smoother, the post-smoother below the finest level). A CTA takes about
+// as long as its planes and two more (halo planes, filling its pipeline) and
+// the CTAs run in waves of two per SM, so the chunk height is the one with the
+// least waves x planes; every node's value is the same for any height. With
+// the 16 planes of the partial sums' layout, 6 samples of 32^3 were 36 CTAs
+// (FP64 pre-smoother: 74 us): a coupled FP64 batch of 6 samples of 128^3 went
+// from 26.9 to 24.3 ms, 16 mixed solves of 64^3 from 3.87 to 3.55 ms (one CTA
+// per SM as a wave: 24.7 and 3.65, three: 24.7 and 3.59).
+constexpr int64_t CHUNK_WAVE = 2 * 152;
+template <class T>
+inline Grid flat_chunks(Grid g, int64_t B) {
+  if (g.zset) return g;
+  // the four-row FP32 kernel takes two 32 x 16 tiles per CTA
+  const int64_t tiles = ((g.n + 31) / 32) * ((g.n + 15) / 16) / (sizeof(T) == 4 && zm_wide(g) && g.zt == 0 ? 2 : 1);
+  const int64_t N1 = g.n + 1;
+  int64_t best = -1;
+  for (int64_t c = 1; 2 * c <= N1; ++c) {
+    const int64_t zc = (N1 + c - 1) / c;
+    if ((N1 + zc - 1) / zc != c) continue;
+    const int64_t t = (tiles * B * c + CHUNK_WAVE - 1) / CHUNK_WAVE * (zc + 2);
+    if (best < 0 || t < best) {
+      best = t;
+      g.zc = (int)zc;
+    }
+  }
+  g.zx = ((g.n + 31) / 32) * ((g.n + 15) / 16) * (int)((N1 + g.zc - 1) / g.zc);
+  return g;
+}
+
 template <int N, class LP, class Epi>
 inline void launch_zm3n_at(cudaStream_t s, const Grid& g, int64_t B, const float* kappa, const LP& lp,
                            const int32_t* active, const Epi& epi, double* part, Prof p) {
@@ -2000,7 +2030,7 @@ namespace d3 {
 
 template <class T>
 cudaError_t apply(cudaStream_t s, const Grid& g, const T* kappa, const T* x, T* y, int64_t B, Prof p) {
-  launch_zm3<T>(s, g, B, kappa, LdX<T>{x, g.ns}, nullptr, EpiApply<T>{y, g.ns}, nullptr, p);
+  launch_zm3<T>(s, flat_chunks<T>(g, B), B, kappa, LdX<T>{x, g.ns}, nullptr, EpiApply<T>{y, g.ns}, nullptr, p);
   return cudaGetLastError();
 }
 template <class T>
@@ -2028,7 +2058,7 @@ cudaError_t mg_pre(cudaStream_t s, const Grid& g, const T* kappa, const T* w, co
   // FP32 levels whose post-smoother forms e = W b again do not store it (mg_post's test)
   const bool keep = !(sizeof(T) == 4 && zm_wide(g) && g.zt == 0 &&
                       (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) == 0);
-  launch_zm3<T>(s, g, B, kappa, LdWb<T>{w, b, g.ns}, active, EpiMgRes<T>{b, r1, keep ? e : nullptr, g.ns}, nullptr, p,
+  launch_zm3<T>(s, flat_chunks<T>(g, B), B, kappa, LdWb<T>{w, b, g.ns}, active, EpiMgRes<T>{b, r1, keep ? e : nullptr, g.ns}, nullptr, p,
                 ks);
   return cudaGetLastError();
 }
@@ -2050,17 +2080,18 @@ template <class T>
 cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* kappa, const T* w,
                     const T* b, const T* e, const T* ec, T* out, T* tmp, const int32_t* active,
                     double* part, int64_t B, Prof p, const T* ks) {
+  const Grid h = part ? g : flat_chunks<T>(g, B);
   if constexpr (std::is_same<T, float>::value) {
     // one kernel (the arrays are a plan's, 256-byte aligned; e is not read)
     if (zm_wide(g) && g.zt == 0 && (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) == 0) {
-      launch_zm3n(s, g, B, kappa, LdPostf{w, b, ec, g.ns, coarse.ns}, active, EpiMgPost<float>{w, b, out, g.ns}, part,
+      launch_zm3n(s, h, B, kappa, LdPostf{w, b, ec, g.ns, coarse.ns}, active, EpiMgPost<float>{w, b, out, g.ns}, part,
                   p);
       return cudaGetLastError();
     }
   }
   k_prolong3<T><<<prolong3_grid(g, B), dim3(32, 8, 1), 0, s>>>(g, coarse.ns, e, ec, tmp, active,
                                                                  Prof{nullptr, 0.0});
-  launch_zm3<T>(s, g, B, kappa, LdX<T>{tmp, g.ns}, active, EpiMgPost<T>{w, b, out, g.ns}, part, p, ks);
+  launch_zm3<T>(s, h, B, kappa, LdX<T>{tmp, g.ns}, active, EpiMgPost<T>{w, b, out, g.ns}, part, p, ks);
   return cudaGetLastError();
 }
 template <class T>

@@ -189,3 +189,24 @@ def test_3d_mixed_workload_finest_level_against_fp64_form(m):
         got[precision] = (qf, qc)
     for a, b in zip(got["mixed"], got["fp64"]):
         assert np.all(np.abs(a - b) <= RTOL_Q * np.abs(b)), (a, b)
+
+
+@pytest.mark.parametrize("n,count", [(2, 700), (9, 200), (32, 60), (40, 20), (64, 7)])
+def test_apply3d_is_the_same_on_every_chunk_height(m, n, count):
+    """A x of one sample alone, in a batch and with the caller's planes per CTA: the same bits, FP64 and FP32."""
+    ns, es, nn = m.node_stride(3, n), m.elem_stride(3, n), (n + 1) ** 3
+    kd = to_dev(random_element_field(3, n, 1, seed=n, spread=1.0), es).repeat(count)
+    xd = to_dev(random_node_vectors(3, n, 1, seed=n + 1), ns).repeat(count)
+    for dtype, call in ((torch.float64, "apply"), (torch.float32, "apply32")):
+        k, x = kd.to(dtype), xd.to(dtype)
+        outs = []
+        for z_chunk, B in ((0, count), (0, 1), (1, 1), (5, 1)):
+            y = torch.zeros(B * ns, dtype=dtype, device="cuda")
+            cfg = m.config(dim=3, n_levels=1, coarse_cells=n)
+            cfg.z_chunk = z_chunk
+            with m.Plan(cfg, stream()) as plan:
+                getattr(plan, call)(0, k.data_ptr(), x.data_ptr(), y.data_ptr(), B)
+                torch.cuda.synchronize()
+            outs.append(y.reshape(B, ns)[:, :nn])
+        for y in outs:
+            assert torch.equal(y, outs[1].expand_as(y))
