@@ -282,7 +282,8 @@ cudaError_t resid64(cudaStream_t s, const Grid& g, const double* kappa, const do
                     const double* ks = nullptr);
 // Per-node kappa sums [K_n | K_x | K_y | K_z] (4 node arrays per sample,
 // sample stride 4 ns) for the FP64 element-sum z-march.
-cudaError_t ksum(cudaStream_t s, const Grid& g, const double* kappa, double* ks, int64_t B);
+cudaError_t ksum(cudaStream_t s, const Grid& g, const double* kappa, double* ks, int64_t B, double omega = 0.0,
+                 double* w = nullptr);
 // nested initial guess: x = P uc (trilinear interpolation from grid `coarse`)
 cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, const double* uc,
                           double* x, const int32_t* active, int64_t B, Prof p);

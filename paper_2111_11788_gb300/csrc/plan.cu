@@ -761,18 +761,18 @@ mlmc_status setup_levels(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
   }
   const double omega = (K > 1) ? p->cfg.mg_omega : 1.0;
   const int kw = std::max(1, K - 1);   // levels that smooth (W = omega / D)
-  // 2D levels with operator coefficients get W from the same kernel; 3D
-  // levels get their kappa sums (FP64) and W separately
+  // levels with operator coefficients (2D) or kappa sums (3D FP64) get W from the same kernel
   const bool d2c = mi.g[0].dim == 2;
   for (int k = 0; k < K; ++k)
     if (w.coef[k])
       CK(run(p, KID_SETUP, [&] {
         if (d2c) return d2::coef<T>(s, mi.g[k], w.kap[k], w.coef[k], B, omega, k < kw ? w.w[k] : nullptr);
-        if constexpr (std::is_same<T, double>::value) return d3::ksum(s, mi.g[k], w.kap[k], w.coef[k], B);
+        if constexpr (std::is_same<T, double>::value) 
+          return d3::ksum(s, mi.g[k], w.kap[k], w.coef[k], B, omega, k < kw ? w.w[k] : nullptr);
         return cudaErrorInvalidValue;
       }));
   for (int k = 0; k < kw; ++k)
-    if (!d2c || !w.coef[k])
+    if (!w.coef[k])
       CK(run(p, KID_SETUP, [&] { return op::winv<T>(s, mi.g[k], w.kap[k], omega, w.w[k], B); }));
   return MLMC_OK;
 }

@@ -528,9 +528,12 @@ __global__ void __launch_bounds__(ZTHREADS, 2) k_zm3q(Grid g, const double* __re
 // Kappa sums of every node (0 outside the mesh), per sample [5 K_n | K_x | K_y
 // | K_z] in node strides: K_n the 8 elements around the node, K_x the 4
 // elements sharing the edge to the +x neighbour (element column i, rows j-1
-// and j, layers k-1 and k), K_y and K_z likewise. Once per solve.
+// and j, layers k-1 and k), K_y and K_z likewise. Once per solve and level. With
+// W also the smoother weights omega / D, D = h/3 K_n (the same values as
+// k_winv3's, without a second pass that sums the 8 elements again: 6 samples of
+// 128^3 644 -> 477 us, bound by the FP64 pipe, the division most of it).
 __global__ void __launch_bounds__(256) k_ksum3(Grid g, const double* __restrict__ K, double* __restrict__ Ks,
-                                               int64_t kss, int pz) {
+                                               int64_t kss, int pz, double omega, double* __restrict__ W) {
   const int64_t b = blockIdx.y;
   const NodeCol c = node_col3(g.n, pz);
   if (!c.valid) return;
@@ -560,6 +563,10 @@ __global__ void __launch_bounds__(256) k_ksum3(Grid g, const double* __restrict_
     kn[g.ns + o] = Y0 + Y1;
     kn[2 * g.ns + o] = X0 + X1;
     kn[3 * g.ns + o] = L1;
+    if (W) {
+      const bool in = c.i > 0 && c.i < n && c.j > 0 && c.j < n && kz > 0 && kz < n;
+      W[b * g.ns + o] = in ? omega / (g.c3 * (L0 + L1)) : 0.0;
+    }
     L0 = L1;
     X0 = X1;
     Y0 = Y1;
@@ -2146,9 +2153,10 @@ cudaError_t resid64(cudaStream_t s, const Grid& g, const double* kappa, const do
   return cudaGetLastError();
 }
 
-cudaError_t ksum(cudaStream_t s, const Grid& g, const double* kappa, double* ks, int64_t B) {
+cudaError_t ksum(cudaStream_t s, const Grid& g, const double* kappa, double* ks, int64_t B, double omega,
+                 double* w) {
   const int pz = node_pz(g.n);
-  k_ksum3<<<dim3(node_col3_blocks(g.n, pz), (unsigned)B, 1), block3(), 0, s>>>(g, kappa, ks, 4 * g.ns, pz);
+  k_ksum3<<<dim3(node_col3_blocks(g.n, pz), (unsigned)B, 1), block3(), 0, s>>>(g, kappa, ks, 4 * g.ns, pz, omega, w);
   return cudaGetLastError();
 }
 
