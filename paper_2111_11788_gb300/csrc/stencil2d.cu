@@ -813,7 +813,7 @@ __global__ void __launch_bounds__(SBLOCK) k_resid2(Grid g, const double* __restr
 template <class T>
 __global__ void __launch_bounds__(FLAT_THREADS) k_coef2(Grid g, const T* __restrict__ K,
                                                         T* __restrict__ Cb, int64_t cs, double omega,
-                                                        T* __restrict__ W) {
+                                                        T* __restrict__ W, int per) {
   const int64_t b = blockIdx.y;
   const int n = g.n, N1 = n + 1;
   const int64_t nn = (int64_t)N1 * N1, ne = (int64_t)n * n;
@@ -822,8 +822,8 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_coef2(Grid g, const T* __restr
   T* ce = cd + g.ns;
   T* cn = cd + 2 * g.ns;
   T* q = cd + 3 * g.ns;
-  const int64_t e0 = (int64_t)blockIdx.x * FLAT_ELEMS;
-  const int64_t e1 = min(e0 + (int64_t)FLAT_ELEMS, g.ns);
+  const int64_t e0 = (int64_t)blockIdx.x * per;
+  const int64_t e1 = min(e0 + per, g.ns);
   for (int64_t e = e0 + threadIdx.x; e < e1; e += FLAT_THREADS) {
     T d = T(0), xe = T(0), xn = T(0);
     if (e < nn) {
@@ -879,6 +879,21 @@ __device__ __forceinline__ void cta_partial(double v, double* __restrict__ part,
 }
 
 inline dim3 fgrid(const Grid& g, int64_t B) { return dim3((unsigned)g.fx, (unsigned)B, 1); }
+
+// Elements per CTA of a pointwise launch without partial sums: FLAT_ELEMS, or
+// less until every SM has its eight CTAs. 16 elements of a thread one after the
+// other were most of the time of a small level: restriction of 30 FP32 samples
+// to 64^2 13.2 us as 60 CTAs, 4.4 as 510; coefficients of 40 FP64 samples of
+// 128^2 53 and 27. fgrid's CTAs, which fix the layout of sums, keep FLAT_ELEMS.
+inline int flat_per(const Grid& g, int64_t B) {
+  int per = FLAT_ELEMS;
+  while (per > FLAT_THREADS && (g.ns + per - 1) / per * B < 8 * 152) per /= 2;
+  return per;
+}
+inline dim3 pgrid(const Grid& g, int64_t B) {
+  const int per = flat_per(g, B);
+  return dim3((unsigned)((g.ns + per - 1) / per), (unsigned)B, 1);
+}
 
 // Nodes of one sample: (n+1)^d. Entries between that and the sample stride
 // are padding that no kernel reads or writes.
@@ -1000,10 +1015,10 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_jz_flat(Grid g, const T* __res
 // x = 0 and, if R != nullptr, r = h^2 at interior nodes (b_i = int phi_i for f = 1).
 template <class T>
 __global__ void __launch_bounds__(FLAT_THREADS) k_init_flat(Grid g, T* __restrict__ X,
-                                                            T* __restrict__ R, Prof prof) {
+                                                            T* __restrict__ R, Prof prof, int per) {
   const int64_t b = blockIdx.y;
-  const int64_t e0 = (int64_t)blockIdx.x * FLAT_ELEMS;
-  const int64_t e1 = min(e0 + (int64_t)FLAT_ELEMS, g.ns);
+  const int64_t e0 = (int64_t)blockIdx.x * per;
+  const int64_t e1 = min(e0 + per, g.ns);
   const int N1 = g.n + 1;
   const int64_t nn = (int64_t)N1 * N1;
   const T h2 = T(g.h * g.h);
@@ -1101,13 +1116,13 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_refine_flat(Grid g, int mode,
 // W = omega / D at every node (0 on the boundary).
 template <class T>
 __global__ void __launch_bounds__(FLAT_THREADS) k_winv2(Grid g, const T* __restrict__ K,
-                                                        double omega, T* __restrict__ W) {
+                                                        double omega, T* __restrict__ W, int per) {
   const int64_t b = blockIdx.y;
   const int N1 = g.n + 1;
   const int64_t nn = (int64_t)N1 * N1;
   const T* k = K + b * g.es;
-  const int64_t e0 = (int64_t)blockIdx.x * FLAT_ELEMS;
-  const int64_t e1 = min(e0 + (int64_t)FLAT_ELEMS, g.ns);
+  const int64_t e0 = (int64_t)blockIdx.x * per;
+  const int64_t e1 = min(e0 + per, g.ns);
   for (int64_t e = e0 + threadIdx.x; e < e1; e += FLAT_THREADS) {
     T w = T(0);
     if (e < nn) {
@@ -1129,15 +1144,15 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_restrict2(Grid gc, int64_t nsf
                                                             const T* __restrict__ R1,
                                                             T* __restrict__ Bc,
                                                             const int32_t* __restrict__ active,
-                                                            Prof prof) {
+                                                            Prof prof, int per) {
   const int64_t b = blockIdx.y;
   if (!active[b]) return;
   const int nc = gc.n;
   const int N1c = nc + 1;
   const int N1 = 2 * nc + 1;
   const int64_t nn = (int64_t)N1c * N1c;
-  const int64_t e0 = (int64_t)blockIdx.x * FLAT_ELEMS;
-  const int64_t e1 = min(e0 + (int64_t)FLAT_ELEMS, gc.ns);
+  const int64_t e0 = (int64_t)blockIdx.x * per;
+  const int64_t e1 = min(e0 + per, gc.ns);
   for (int64_t e = e0 + threadIdx.x; e < e1; e += FLAT_THREADS) {
     T v = T(0);
     if (e < nn) {
@@ -1157,7 +1172,7 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_restrict2(Grid gc, int64_t nsf
 }
 
 // The same full weighting on warp strips (the FP64 form): a warp owns 32
-// coarse columns I (one per lane) and walks RSTRIP_ROWS coarse rows J. On
+// coarse columns I (one per lane) and walks ROWS coarse rows J. On
 // each fine row a lane loads one aligned pair of fine values, (2I, 2I + 1) on
 // even rows and (2I - 1, 2I) on odd rows (fine rows have an odd length, so on
 // odd rows the pair starting at 2I - 1 is the aligned one), and takes the
@@ -1165,7 +1180,7 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_restrict2(Grid gc, int64_t nsf
 // 0 and 31 load theirs); the sum over the odd fine row 2J + 1 is carried to
 // coarse row J + 1, so each fine value is read once (twice on the first row
 // of a chunk). Every node of the coarse rows is written (0 off the interior).
-constexpr int RSTRIP_ROWS = 16;
+constexpr int RSTRIP_ROWS = 16, RSTRIP_SHORT = 4;
 template <class T>
 struct Vec2;
 template <>
@@ -1177,7 +1192,7 @@ struct Vec2<double> {
   using V = double2;
 };
 
-template <class T>
+template <class T, int ROWS>
 __global__ void __launch_bounds__(SBLOCK) k_restrict2s(Grid gc, int64_t nsf, const T* __restrict__ R1,
                                                        T* __restrict__ Bc, const int32_t* __restrict__ active,
                                                        Prof prof) {
@@ -1191,7 +1206,7 @@ __global__ void __launch_bounds__(SBLOCK) k_restrict2s(Grid gc, int64_t nsf, con
   const int I0 = (blockIdx.x * SWARPS + (threadIdx.x >> 5)) * 32;
   if (I0 > nc) return;   // the whole strip lies beyond the row
   const int I = I0 + lane;
-  const int J0 = blockIdx.y * RSTRIP_ROWS, J1 = min(J0 + RSTRIP_ROWS, N1c);
+  const int J0 = blockIdx.y * ROWS, J1 = min(J0 + ROWS, N1c);
   const T* __restrict__ r = R1 + b * nsf;
   T* __restrict__ bc = Bc + b * gc.ns;
   const T h = T(0.5);
@@ -1329,14 +1344,14 @@ cudaError_t apply(cudaStream_t s, const Grid& g, const T* kappa, const T* x, T* 
 
 template <class T>
 cudaError_t winv(cudaStream_t s, const Grid& g, const T* kappa, double omega, T* w, int64_t B) {
-  k_winv2<T><<<fgrid(g, B), FLAT_THREADS, 0, s>>>(g, kappa, omega, w);
+  k_winv2<T><<<pgrid(g, B), FLAT_THREADS, 0, s>>>(g, kappa, omega, w, flat_per(g, B));
   return cudaGetLastError();
 }
 
 template <class T>
 cudaError_t pcg_init(cudaStream_t s, const Grid& g, T* x, T* r, int64_t B, Prof p) {
   if (r)
-    k_init_flat<T><<<fgrid(g, B), FLAT_THREADS, 0, s>>>(g, x, r, p);
+    k_init_flat<T><<<pgrid(g, B), FLAT_THREADS, 0, s>>>(g, x, r, p, flat_per(g, B));
   else
     k_zero_flat<T><<<fgrid(g, B), FLAT_THREADS, 0, s>>>(g, x, p);
   return cudaGetLastError();
@@ -1353,7 +1368,7 @@ inline int64_t coef_stride(const Grid& g) { return 3 * g.ns + g.es; }
 
 template <class T>
 cudaError_t coef(cudaStream_t s, const Grid& g, const T* kappa, T* coef, int64_t B, double omega, T* w) {
-  k_coef2<T><<<fgrid(g, B), FLAT_THREADS, 0, s>>>(g, kappa, coef, coef_stride(g), omega, w);
+  k_coef2<T><<<pgrid(g, B), FLAT_THREADS, 0, s>>>(g, kappa, coef, coef_stride(g), omega, w, flat_per(g, B));
   return cudaGetLastError();
 }
 
@@ -1404,12 +1419,17 @@ cudaError_t restrict_(cudaStream_t s, const Grid& fine, const Grid& coarse, cons
   // node, whose independent loads hide the latency of the mostly L2-resident
   // FP32 arrays better (the strips took 31% longer there).
   if constexpr (sizeof(T) == 8) {
-    const int N1c = coarse.n + 1;
-    const dim3 grid((unsigned)((N1c + 32 * SWARPS - 1) / (32 * SWARPS)),
-                    (unsigned)((N1c + RSTRIP_ROWS - 1) / RSTRIP_ROWS), (unsigned)B);
-    k_restrict2s<T><<<grid, SBLOCK, 0, s>>>(coarse, fine.ns, r1, bc, active, p);
+    // chunks of RSTRIP_ROWS coarse rows, or of RSTRIP_SHORT where the tall ones
+    // do not give every SM partition four warps (40 samples to 128^2: 17.1 ->
+    // 12.6 us, to 64^2: 13.7 -> 6.8)
+    const int N1c = coarse.n + 1, strips = (N1c + 31) / 32, gx = (strips + SWARPS - 1) / SWARPS;
+    auto grid = [&](int rows) { return dim3((unsigned)gx, (unsigned)((N1c + rows - 1) / rows), (unsigned)B); };
+    if ((int64_t)strips * ((N1c + RSTRIP_ROWS - 1) / RSTRIP_ROWS) * B < 4 * 4 * 152)
+      k_restrict2s<T, RSTRIP_SHORT><<<grid(RSTRIP_SHORT), SBLOCK, 0, s>>>(coarse, fine.ns, r1, bc, active, p);
+    else
+      k_restrict2s<T, RSTRIP_ROWS><<<grid(RSTRIP_ROWS), SBLOCK, 0, s>>>(coarse, fine.ns, r1, bc, active, p);
   } else {
-    k_restrict2<T><<<fgrid(coarse, B), FLAT_THREADS, 0, s>>>(coarse, fine.ns, r1, bc, active, p);
+    k_restrict2<T><<<pgrid(coarse, B), FLAT_THREADS, 0, s>>>(coarse, fine.ns, r1, bc, active, p, flat_per(coarse, B));
   }
   return cudaGetLastError();
 }

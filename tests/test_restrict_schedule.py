@@ -118,3 +118,10 @@ def test_strip_restriction_is_the_transpose_of_bilinear_prolongation(nc):
     need = {(fr, fc) for fr in range(1, n) for fc in range(1, n)}
     if nc >= 2:
         assert need <= set(reads)
+
+
+@pytest.mark.parametrize("nc", [1, 2, 31, 32, 64])
+def test_the_same_on_shorter_chunks(monkeypatch, nc):
+    """Batches that leave SM partitions idle use chunks of 4 coarse rows."""
+    monkeypatch.setitem(globals(), "RSTRIP_ROWS", 4)
+    test_strip_restriction_is_the_transpose_of_bilinear_prolongation(nc)
