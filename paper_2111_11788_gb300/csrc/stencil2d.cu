@@ -427,25 +427,39 @@ __device__ __forceinline__ void warp_partial(T v, double* __restrict__ part, int
 
 inline dim3 sgrid(const Grid& g, int64_t B) { return dim3((unsigned)g.sx, (unsigned)g.sy, (unsigned)B); }
 
-// Rows per strip of a launch that leaves no partial sums (A x, the pre-smoother,
-// the post-smoother below the finest level): SROWS, or SROWS_SHORT where the
-// tall strips are fewer warps than the SMs have partitions. A row costs about
+// Rows per strip of a launch that leaves no partial sums (A x, the pre-
+// smoother, the post-smoother below the finest level): the height of the least
+// waves x rows. A wave is one warp per SM partition in FP64 (the FP64 pipe
+// takes no more) and eight in FP32 (bound by latency until then), and a strip
+// takes as long as its rows and one or two more (its halo). A row costs about
 // 0.8 us of dependent FP64 and L2 latency, which a launch of few warps cannot
 // hide (A x of one sample of 45^2: 22.5 us on 32-row strips, 6.1 us on 4-row
-// ones, launch and binding included); every node's value is the same for
-// either height. The height is a template parameter: as a field of the grid it
-// cost 8 to 16 registers a thread and 4% of a batch of 40 samples of 256^2.
-// Launches with partial sums keep SROWS, which fixes the sums' layout.
-constexpr int SROWS_SHORT = 4;
-constexpr int64_t STRIP_WARPS = 4 * 152;
-template <class F>
+// ones, launch and binding included; FP64 post-smoother of 40 samples of 128^2:
+// 43.6 and 28.9 on 16 rows; FP32 pre-smoother of 30 samples of 128^2: 13.5 and
+// 6.4 on 8 rows; 16 FP64 solves of 512^2: 7.6 and 6.6 ms); every node's value
+// is the same for any height. The height is a template parameter: as a field of
+// the grid it cost 8 to 16 registers a thread and 4% of a batch of 40 samples
+// of 256^2. Launches with partial sums keep SROWS, which fixes the sums'
+// layout.
+template <class T, class F>
 void with_strips(const Grid& g, int64_t B, F&& launch) {
-  const int64_t columns = (int64_t)g.sx * SWARPS * B;
-  if (columns * g.sy < STRIP_WARPS)
-    launch(std::integral_constant<int, SROWS_SHORT>{},
-           dim3((unsigned)g.sx, (unsigned)((g.n + SROWS_SHORT) / SROWS_SHORT), (unsigned)B));
-  else
-    launch(std::integral_constant<int, SROWS>{}, sgrid(g, B));
+  constexpr bool f64 = sizeof(T) == 8;
+  constexpr int64_t wave = 4 * 152 * (f64 ? 1 : 8);
+  const int64_t strips = (g.n + 1 + 29) / 30 * B;
+  int best = SROWS;
+  int64_t best_t = INT64_MAX;
+  for (int rows = SROWS; rows >= 4; rows /= 2) {
+    const int64_t t = (strips * ((g.n + rows) / rows) + wave - 1) / wave * (rows + (f64 ? 1 : 2));
+    if (t < best_t) {
+      best_t = t;
+      best = rows;
+    }
+  }
+  const dim3 grid((unsigned)g.sx, (unsigned)((g.n + best) / best), (unsigned)B);
+  if (best == 4) launch(std::integral_constant<int, 4>{}, grid);
+  else if (best == 8) launch(std::integral_constant<int, 8>{}, grid);
+  else if (best == 16) launch(std::integral_constant<int, 16>{}, grid);
+  else launch(std::integral_constant<int, SROWS>{}, grid);
 }
 constexpr int SBLOCK = SWARPS * 32;
 
@@ -1336,7 +1350,7 @@ cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, con
 
 template <class T>
 cudaError_t apply(cudaStream_t s, const Grid& g, const T* kappa, const T* x, T* y, int64_t B, Prof p) {
-  with_strips(g, B, [&](auto sr, dim3 grid) {
+  with_strips<T>(g, B, [&](auto sr, dim3 grid) {
     k_apply2<T, decltype(sr)::value><<<grid, SBLOCK, 0, s>>>(g, kappa, x, y, p);
   });
   return cudaGetLastError();
@@ -1401,7 +1415,7 @@ cudaError_t jacobi_z(cudaStream_t s, const Grid& g, const T* winv, const T* r, T
 template <class T>
 cudaError_t mg_pre(cudaStream_t s, const Grid& g, const T* kappa, const T* w, const T* b, T* e,
                    T* r1, const int32_t* active, int64_t B, Prof p, const T* coef) {
-  with_strips(g, B, [&](auto sr, dim3 grid) {
+  with_strips<T>(g, B, [&](auto sr, dim3 grid) {
     constexpr int SR = decltype(sr)::value;
     if (coef)
       k_mgpre2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coef, coef_stride(g), w, b, e, r1, active, p);
@@ -1459,7 +1473,7 @@ cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* 
   if (part)
     launch(std::integral_constant<int, SROWS>{}, sgrid(g, B));
   else
-    with_strips(g, B, launch);
+    with_strips<T>(g, B, launch);
   return cudaGetLastError();
 }
 
