@@ -37,7 +37,8 @@ constexpr int RES_THREADS = 256;
 constexpr int RES_PER_SM = 3;     // CTAs per SM the registers allow
 
 constexpr int RES_BAND = 512;     // interior nodes from which a mesh gets another band
-constexpr int RES_MAX_V = 8;      // bands of a sample, hence CTAs (a portable cluster)
+constexpr int RES_MAX_V = 16;     // bands of a sample, hence CTAs of its cluster
+constexpr int RES_PORTABLE = 8;   // CTAs of a portable cluster
 constexpr int RES_MAX_LEVELS = MAX_RESIDENT_LEVELS;   // 128 .. 2 cells
 constexpr size_t RES_SMEM_MAX = 224 * 1024;
 constexpr size_t RES_SMEM_SHARE = 74 * 1024;   // shared memory of a CTA at RES_PER_SM of them
@@ -65,7 +66,8 @@ struct ResLevel {
 template <class T>
 struct ResArgs {
   int K, C, nd;        // multigrid levels; CTAs per sample; levels split over the CTAs
-  int V, nv, Rv;       // level 0: bands the sums are formed in, bands per CTA, slabs per band
+  int V, nv, Rv;       // level 0: bands the sums are formed in, bands per CTA, slabs per band (most of them)
+  int shv;             // log2 V
   ResLevel<T> lv[RES_MAX_LEVELS];
   unsigned ox, op, oz, ored, osw, osc;   // x, p, zeros, sums, scalars
   unsigned bytes;
@@ -98,10 +100,22 @@ struct Res {
   int64_t smp;
   int tid;
   int slot;
+  int f0, c0;   // level 0: this CTA's first slab and its slabs
 
   __device__ __forceinline__ bool mine(int l) const { return l < a.nd || rank == 0; }
-  __device__ __forceinline__ int first(int l) const { return l < a.nd || l == 0 ? rank * a.lv[l].R + 1 : 1; }
+  // the slabs of level 0 before band v: bands of Rv slabs where levels meet, else
+  // (one level, any n) even shares of the n - 1 slabs
+  __device__ __forceinline__ int edge(int v) const {
+    const int m = a.lv[0].n - 1;
+    return a.K == 1 ? (v * m) >> a.shv : min(v * a.Rv, m);
+  }
+  __device__ __forceinline__ void deal() {
+    f0 = edge(rank * a.nv) + 1;
+    c0 = edge((rank + 1) * a.nv) + 1 - f0;
+  }
+  __device__ __forceinline__ int first(int l) const { return l == 0 ? f0 : l < a.nd ? rank * a.lv[l].R + 1 : 1; }
   __device__ __forceinline__ int own(int l) const {
+    if (l == 0) return c0;
     const int n = a.lv[l].n;
     return max(0, min(a.lv[l].R, n - first(l)));
   }
@@ -134,7 +148,8 @@ struct Res {
   template <class V>
   __device__ __forceinline__ const V* before(int l, unsigned off) const {
     if (l >= a.nd || rank == 0) return at<V>(a.oz);
-    return remote(at<V>(off) + (a.lv[l].R - 1) * a.lv[l].S, rank - 1);
+    const int last = (a.K == 1 ? f0 - 1 - edge((rank - 1) * a.nv) : a.lv[l].R) - 1;
+    return remote(at<V>(off) + last * a.lv[l].S, rank - 1);
   }
   template <class V>
   __device__ __forceinline__ const V* after(int l, unsigned off) const {
@@ -170,9 +185,11 @@ struct Res {
   // per band, in an order that does not depend on how many bands a CTA has.
   template <class F, class D>
   __device__ __forceinline__ void nodes0(F&& f, D&& done) const {
-    for (int v = 0; v < a.nv; ++v) {
-      slab_nodes(0, v * a.Rv, max(0, min(a.Rv, own(0) - v * a.Rv)), f);
+    for (int v = 0, s0 = 0; v < a.nv; ++v) {
+      const int s1 = edge(rank * a.nv + v + 1) + 1 - f0;
+      slab_nodes(0, s0, s1 - s0, f);
       done(v);
+      s0 = s1;
     }
   }
   // f - (A v) at node (o, i, j) of slab z, v given by the slabs around it
@@ -252,10 +269,15 @@ struct Res {
       const T* vp = js < cnt - 1 ? v0 + S : hi;
       f(js * S + o, (z0 + js) * S + o, resid<T>(n, L.ns, L.d0, L.d1, kap, coef, vm, v0, vp, z0 + js, o, i, j, rhs(js * S + o)));
     };
-    const int nb = l == 0 ? a.nv : 1, per = l == 0 ? a.Rv : cnt;
-    for (int b = 0; b < nb; ++b) {
-      slab_nodes(l, b * per, max(0, min(per, cnt - b * per)), node);
-      if (l == 0) done(b);
+    if (l > 0) {
+      slab_nodes(l, 0, cnt, node);
+      return;
+    }
+    for (int v = 0, s0 = 0; v < a.nv; ++v) {
+      const int s1 = edge(rank * a.nv + v + 1) + 1 - f0;
+      slab_nodes(l, s0, s1 - s0, node);
+      done(v);
+      s0 = s1;
     }
   }
   // Sums over the sample: every thread hands in its part of each of its CTA's
@@ -633,7 +655,8 @@ __global__ void __launch_bounds__(RES_THREADS, RES_PER_SM) k_resident(const __gr
   extern __shared__ __align__(16) unsigned char res_sm[];
   const int tid = threadIdx.x;
   for (int64_t smp = blockIdx.x / a.C; smp < a.B; smp += gridDim.x / a.C) {
-    Res<DIM, T, MIXED> s{a, res_sm, (int)(blockIdx.x % a.C), smp, tid, 0};
+    Res<DIM, T, MIXED> s{a, res_sm, (int)(blockIdx.x % a.C), smp, tid, 0, 0, 0};
+    s.deal();
     for (unsigned k = tid; k < a.bytes / 8; k += RES_THREADS) reinterpret_cast<double*>(res_sm)[k] = 0.0;
     s.all_sync();   // the cluster has started and every array is zero
     if constexpr (MIXED) s.solve_mixed();
@@ -653,7 +676,8 @@ __global__ void __launch_bounds__(RES_THREADS, RES_PER_SM) k_bottom(const __grid
                                                                     Prof prof) {
   extern __shared__ __align__(16) unsigned char res_sm[];
   const int tid = threadIdx.x;
-  Res<DIM, T, false> s{a, res_sm, (int)(blockIdx.x % a.C), (int64_t)(blockIdx.x / a.C), tid, 0};
+  Res<DIM, T, false> s{a, res_sm, (int)(blockIdx.x % a.C), (int64_t)(blockIdx.x / a.C), tid, 0, 0, 0};
+  s.deal();
   if (!active[s.smp]) return;   // the whole cluster
   for (unsigned k = tid; k < a.bytes / 8; k += RES_THREADS) reinterpret_cast<double*>(res_sm)[k] = 0.0;
   __syncthreads();
@@ -807,6 +831,8 @@ static size_t resident_layout(int dim, int n, int K, int V, int C, ResArgs<T>& a
   a.V = V;
   a.nv = V / C;
   a.Rv = K > 1 ? std::max(1, n / V) : (n - 1 + V - 1) / V;
+  a.shv = 0;
+  while ((1 << a.shv) < V) ++a.shv;
   a.nd = 0;
   int64_t band0 = 0;
   for (int l = 0; l < K; ++l) {
@@ -818,7 +844,7 @@ static size_t resident_layout(int dim, int n, int K, int V, int C, ResArgs<T>& a
     // a block's worth of work (2D above 16 rows, 3D above 4 planes)
     const bool split = C > 1 && a.nd == l && (l == 0 || (L.n >= C && L.n > (dim == 2 ? 16 : 4)));
     if (split) a.nd = l + 1;
-    L.R = split ? (K > 1 ? std::max(1, L.n / C) : a.Rv * a.nv) : L.n - 1;
+    L.R = split ? (K > 1 ? std::max(1, L.n / C) : (a.nv * (n - 1) + V - 1) / V) : L.n - 1;
     L.sh = 0;
     while (K > 1 && (1 << (L.sh + 1)) <= L.R) ++L.sh;
     const uint64_t m = (uint64_t)std::max(1, L.n - 1), two32 = (uint64_t)1 << 32;
@@ -856,14 +882,21 @@ static size_t resident_bytes(int dim, int n, int K, int V, int C, bool mixed) {
 // levels (1: Jacobi), or 0 where it does not run: one per 512 interior nodes,
 // at most a portable cluster, where a band of every vector fits a CTA's
 // shared memory. 3D FP64 stops at 16^3 cells (Jacobi: 32^3): there the
-// element-sum z-march does half the FP64 operations per node.
+// element-sum z-march does half the FP64 operations per node. Jacobi, whose
+// hundreds of iterations are one stencil and two sums each, goes on to 16: one
+// sample of 100^2 3.86 -> 2.93 ms, 20 samples 5.49 -> 4.64 (100 samples, two
+// bands a CTA, 14.2 -> 14.8). With multigrid the second band of a CTA cost the
+// large batches of 32^3 5%, so it stays at 8.
 int resident_bands(int dim, int n, int K, bool mixed) {
   if (n < 2 || K < 1 || K > RES_MAX_LEVELS) return 0;
   if (n > (dim == 2 ? 256 : mixed ? 40 : K > 1 ? 16 : 32)) return 0;
   const int64_t in = ipow(n - 1, dim);
   int V = 1;
-  while (V < RES_MAX_V && in > (int64_t)V * RES_BAND && 2 * V <= n) V *= 2;
-  return resident_bytes(dim, n, K, V, V, mixed) <= RES_SMEM_MAX ? V : 0;
+  while (V < RES_PORTABLE && in > (int64_t)V * RES_BAND && 2 * V <= n) V *= 2;
+  if (resident_bytes(dim, n, K, V, V, mixed) > RES_SMEM_MAX) return 0;
+  const bool more = K == 1 && V == RES_PORTABLE && in > (int64_t)V * RES_BAND && RES_MAX_V <= n &&
+                    resident_bytes(dim, n, K, RES_MAX_V, RES_PORTABLE, mixed) <= RES_SMEM_MAX;
+  return more ? RES_MAX_V : V;
 }
 
 // CTAs per sample for a batch: one per band while the batch leaves room on the
@@ -871,7 +904,9 @@ int resident_bands(int dim, int n, int K, bool mixed) {
 // bands in turn, in the same order of sums).
 static int resident_ctas(int dim, int n, int K, int V, bool mixed, int64_t B, int64_t slots) {
   int C = V;
-  while (C > 1 && B * C > slots && resident_bytes(dim, n, K, V, C / 2, mixed) <= RES_SMEM_SHARE) C /= 2;
+  while (C > 1 && B * C > slots &&
+         (C > RES_PORTABLE || resident_bytes(dim, n, K, V, C / 2, mixed) <= RES_SMEM_SHARE))
+    C /= 2;
   return C;
 }
 
@@ -879,8 +914,11 @@ template <int DIM, class T, bool MIXED>
 static cudaError_t launch_res(cudaStream_t s, const ResArgs<T>& a, int64_t B) {
   static std::atomic<uint64_t> opted{0};
   cudaError_t e = once_per_device(opted, [] {
-    return cudaFuncSetAttribute(k_resident<DIM, T, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)RES_SMEM_MAX);
+    const cudaError_t e1 = cudaFuncSetAttribute(k_resident<DIM, T, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)RES_SMEM_MAX);
+    return e1 != cudaSuccess ? e1
+                             : cudaFuncSetAttribute(k_resident<DIM, T, MIXED>,
+                                                    cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -1019,7 +1057,7 @@ cudaError_t launch_bottom(cudaStream_t s, const BottomLevels<T>& lv, const T* b,
   // over a sample here, so the result does not depend on it), at least as
   // many as its arrays need
   int C = 1;
-  while (C < RES_MAX_V && ipow(n - 1, dim) > (int64_t)C * RES_THREADS && 2 * C <= n) C *= 2;
+  while (C < RES_PORTABLE && ipow(n - 1, dim) > (int64_t)C * RES_THREADS && 2 * C <= n) C *= 2;
   ResArgs<T> a{};
   while (C > 1 && B * C > RES_SLOTS && resident_layout(dim, n, lv.L, C / 2, C / 2, a, false) <= RES_SMEM_SHARE) C /= 2;
   if (resident_layout(dim, n, lv.L, C, C, a, false) > RES_SMEM_MAX) return cudaErrorInvalidValue;

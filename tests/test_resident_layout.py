@@ -6,7 +6,7 @@ need. Every interior node is visited once, and every slab a CTA reads lies in
 the band of the CTA it is read from, or is the slab of zeros."""
 import pytest
 
-THREADS, BAND, MAX_V, MAX_LEVELS, SMEM, SHARE = 256, 512, 8, 7, 224 * 1024, 74 * 1024
+THREADS, BAND, MAX_V, PORTABLE, MAX_LEVELS, SMEM, SHARE = 256, 512, 16, 8, 7, 224 * 1024, 74 * 1024
 
 
 def layout(dim, n, K, V, C, mixed, solve=True):
@@ -27,7 +27,7 @@ def layout(dim, n, K, V, C, mixed, solve=True):
         split = C > 1 and nd == l and (l == 0 or (nl >= C and nl > (16 if dim == 2 else 4)))
         if split:
             nd = l + 1
-        R = (max(1, nl // C) if K > 1 else rv * nv) if split else nl - 1
+        R = (max(1, nl // C) if K > 1 else -(-nv * (n - 1) // V)) if split else nl - 1
         m = max(1, nl - 1)
         lv.append(dict(n=nl, N1=N1, S=S, R=R, m1=-(-2 ** 32 // m) % 2 ** 32, m2=-(-2 ** 32 // (m * m)) % 2 ** 32))
         for _ in range((0 if K > 1 and l == K - 1 else 2) + (1 if K > 1 else 0)):
@@ -39,7 +39,8 @@ def layout(dim, n, K, V, C, mixed, solve=True):
         take(4 * 2 * MAX_V, 8)
         take((1 if K > 1 else 2) * nv * THREADS, 8)
         take(48, 1)
-    lv[0]["rv"] = rv
+    lv[0]["edge"] = [v * (n - 1) // V if K == 1 else min(v * rv, n - 1) for v in range(V + 1)]
+    lv[0]["nv"] = nv
     return lv, nd, (off + 15) // 16 * 16
 
 
@@ -47,15 +48,22 @@ def bands(dim, n, K, mixed):
     if n < 2 or K > MAX_LEVELS or n > (256 if dim == 2 else 40 if mixed else 16 if K > 1 else 32):
         return 0
     V = 1
-    while V < MAX_V and (n - 1) ** dim > V * BAND and 2 * V <= n:
+    while V < PORTABLE and (n - 1) ** dim > V * BAND and 2 * V <= n:
         V *= 2
-    return V if layout(dim, n, K, V, V, mixed)[2] <= SMEM else 0
+    if layout(dim, n, K, V, V, mixed)[2] > SMEM:
+        return 0
+    more = K == 1 and V == PORTABLE and (n - 1) ** dim > V * BAND and n >= MAX_V and \
+        layout(dim, n, K, MAX_V, PORTABLE, mixed)[2] <= SMEM
+    return MAX_V if more else V
 
 
 def band(lv, nd, C, l, rank):
     """(first slab, slabs) of a CTA on level l."""
     if l >= nd and rank:
         return 1, 0
+    if l == 0:
+        edge, nv = lv[0]["edge"], lv[0]["nv"]
+        return edge[rank * nv] + 1, edge[(rank + 1) * nv] - edge[rank * nv]
     z0 = rank * lv[l]["R"] + 1 if l < nd else 1
     return z0, max(0, min(lv[l]["R"], lv[l]["n"] - z0))
 
@@ -76,7 +84,7 @@ def test_bands_slabs_and_shared_memory(dim, n, K, mixed):
     while C >= 1:
         check(dim, n, K, mixed, V, C)
         C //= 2
-        if C and layout(dim, n, K, V, C, mixed)[2] > SHARE:
+        if C and C < PORTABLE and layout(dim, n, K, V, C, mixed)[2] > SHARE:
             break
 
 
@@ -84,8 +92,8 @@ def check(dim, n, K, mixed, V, C):
     lv, nd, bytes_ = layout(dim, n, K, V, C, mixed)
     assert bytes_ <= SMEM and nd <= max(1, K - 1) and (C == 1) == (nd == 0)
     # the bands of the sums: rv slabs each, together every slab of level 0, V / C per CTA
-    rv = lv[0]["rv"]
-    assert V * rv >= n - 1 and (V == 1 or C == 1 or rv * (V // C) == lv[0]["R"])
+    edge = lv[0]["edge"]
+    assert edge[0] == 0 and edge[V] == n - 1 and all(a < b or (K > 1 and b == n - 1) for a, b in zip(edge, edge[1:]))
     for l, L in enumerate(lv):
         nl, m, R, S = L["n"], L["n"] - 1, L["R"], L["S"]
         if K > 1 and l < nd:
@@ -117,15 +125,17 @@ def check(dim, n, K, mixed, V, C):
             if z <= 0 or z >= nl:
                 return None
             return ((z - 1) // R, (z - 1) % R) if l < nd else (0, z - 1)
-        for z in range(1, nl):
-            assert slab(z) == owner[z]
+        if K > 1:   # one level alone has no transfers: its bands are even shares, read by before and after only
+            for z in range(1, nl):
+                assert slab(z) == owner[z]
         for r in range(C):
             z0, own = band(lv, nd, C, l, r)
             if own == 0:
                 continue
             # the slabs before and after the band: the last of CTA r - 1, the first of CTA r + 1
-            assert slab(z0 - 1) == (None if r == 0 or l >= nd else (r - 1, R - 1))
-            assert slab(z0 + own) == (None if z0 + own >= nl else (r + 1, 0))
+            last = (band(lv, nd, C, 0, r - 1)[1] if l == 0 and r else R) - 1
+            assert owner.get(z0 - 1) == (None if r == 0 or l >= nd else (r - 1, last))
+            assert owner.get(z0 + own) == (None if z0 + own >= nl else (r + 1, 0))
         if K > 1 and l + 1 < K:
             nc = lv[l + 1]["n"]
             for z in range(1, nc):       # full weighting reads fine slabs 2z - 1 .. 2z + 1, columns 2I - 1 .. 2I + 1
@@ -142,7 +152,7 @@ BOTTOM_SLOTS = 152 * 3
 def test_bottom_levels_fit_every_batch(dim, n, K, mixed):
     """The V-cycle's fused levels: the CTAs a batch gives a sample, each with room for its arrays."""
     top = 1
-    while top < MAX_V and (n - 1) ** dim > top * THREADS and 2 * top <= n:
+    while top < PORTABLE and (n - 1) ** dim > top * THREADS and 2 * top <= n:
         top *= 2
     for B in (1, 40, 57, 58, 100, 500, 60000):
         C = top
