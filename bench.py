@@ -507,9 +507,9 @@ def serving_run(m, args, device=0, adapt=0):
 # 3D (element-sum z-march on precomputed kappa sums, k_zm3q): per element
 # position 3 adds (plane sum of its 4 nodes), 1 add and 1 multiply (Q =
 # kappa S); per node 1.5 adds (x pairs of Q, shared by the two rows of a
-# thread) + 1 add (2 x 2 sum of Q) + 1 multiply and 5 FMAs (six face
-# neighbours) + 1 multiply and 1 FMA (5 u K_n) + 2 adds (minus the two
-# layers' sums): 17.5 instructions, 23.5 flops for the operator. Loaders and
+# thread) + 1 add (2 x 2 sum of Q) + 1 add (the two layers' sums, negated,
+# which start the chain) + 6 FMAs (six face neighbours) + 1 FMA (u times 5 K_n,
+# stored): 15.5 instructions, 22.5 flops for the operator. Loaders and
 # epilogues: A p: z + beta p (1 FMA), q = h/12 t (1 multiply), p.q (1 FMA);
 # pre-smoother: W b (1 multiply), b - h/12 t (1 FMA); post-smoother: b -
 # h/12 t, e + W r and b.out (3 FMAs); residual: f - h/12 t and r.r (2 FMAs).
@@ -519,8 +519,8 @@ def serving_run(m, args, device=0, adapt=0):
 FP64_WORK = {
     (2, "mg_post"): (13.0, 25.0, 42.0), (2, "mg_pre"): (10.0, 19.0, 40.0),
     (2, "pcg_pq"): (11.0, 21.0, 40.0), (2, "resid64"): (10.0, 20.0, 24.0),
-    (3, "mg_post"): (20.5, 29.5, 41.0), (3, "mg_pre"): (19.5, 26.5, 40.0),
-    (3, "pcg_pq"): (20.5, 28.5, 40.0), (3, "resid64"): (19.5, 27.5, 24.0),
+    (3, "mg_post"): (18.5, 28.5, 41.0), (3, "mg_pre"): (17.5, 25.5, 40.0),
+    (3, "pcg_pq"): (18.5, 27.5, 40.0), (3, "resid64"): (17.5, 26.5, 24.0),
 }
 # DRAM bytes per output node measured by ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch whose arrays exceed L2), for the

@@ -700,12 +700,14 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
   while (k0 - 1 >= 1 && mi.g[k0 - 1].n <= nmax) --k0;
   const bool fuse = k0 < K - 1 && K - k0 <= MAX_BOTTOM;
   const int kd = fuse ? k0 : K - 1;   // levels above the bottom
+  // node arrays a smoother moves: FP32 forms e = W b again instead of keeping it (3D: on the four-row tiles)
+  const double na = sizeof(T) == 4 && (g0.dim == 2 || g0.zt == 0) ? 3.0 : 4.0;
   for (int k = 0; k < kd; ++k) {
     const Grid& g = mi.g[k];
     const double nn = nodes_of(g), ne = elems_of(g);
     CK(run(p, KID_MG_PRE, [&] {
       return op::mg_pre<T>(s, g, w.kap[k], w.w[k], w.bk[k], w.e[k], w.r1[k], w.sc.active, B,
-                           prof_for(p, KID_MG_PRE, (4 * nn + ne) * vb), w.coef[k]);
+                           prof_for(p, KID_MG_PRE, (na * nn + ne) * vb), w.coef[k]);
     }));
     CK(run(p, KID_RESTRICT, [&] {
       return op::restrict_<T>(s, g, mi.g[k + 1], w.r1[k], w.bk[k + 1], w.sc.active, B,
@@ -740,7 +742,7 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
       // r1[k] is dead once restricted: it serves as the 3D scratch for e + P e_c
       return op::mg_post<T>(s, g, mi.g[k + 1], w.kap[k], w.w[k], w.bk[k], w.e[k], w.eo[k + 1],
                             w.eo[k], w.r1[k], w.sc.active, k == 0 ? w.part : nullptr, B,
-                            prof_for(p, KID_MG_POST, (4 * nn + ne + nc) * vb), w.coef[k]);
+                            prof_for(p, KID_MG_POST, (na * nn + ne + nc) * vb), w.coef[k]);
     }));
   }
   *tiles = g0.tiles_s;
