@@ -85,10 +85,12 @@ typedef struct mlmc_config {
                               k_x + k_y (+ k_z) <= K (each k < m), M of them, in
                               the full basis' flat order */
   int32_t z_chunk;         /* 3D: z-planes per stencil CTA (0 = built-in rule:
-                              all planes up to 24, else 16); set by mlmc_autotune */
+                              all planes up to 24, else 16, and by the batch
+                              where no sums are formed); set by mlmc_autotune */
   int32_t nested_guess;    /* 1 (default): in a coupled batch of level l > 0 the
                               mesh l-1 solve runs first and its solution,
-                              interpolated (bi/trilinear) to mesh l, is the
+                              interpolated to mesh l (cubic along each axis,
+                              linear where mesh l-1 has few cells), is the
                               initial iterate of the mesh l solve; 0: both
                               solves start from u = 0. The stopping test
                               (||r|| <= rtol ||b||) is the same either way. */
