@@ -650,8 +650,11 @@ struct Res {
   }
 };
 
+// 2D: 64 registers without spills, a fourth CTA on an SM where its shared memory
+// fits (300 mixed samples of 128^2: 3.82 -> 3.01 ms)
 template <int DIM, class T, bool MIXED>
-__global__ void __launch_bounds__(RES_THREADS, RES_PER_SM) k_resident(const __grid_constant__ ResArgs<T> a) {
+__global__ void __launch_bounds__(RES_THREADS, DIM == 2 ? RES_PER_SM + 1 : RES_PER_SM)
+    k_resident(const __grid_constant__ ResArgs<T> a) {
   extern __shared__ __align__(16) unsigned char res_sm[];
   const int tid = threadIdx.x;
   for (int64_t smp = blockIdx.x / a.C; smp < a.B; smp += gridDim.x / a.C) {
@@ -879,24 +882,24 @@ static size_t resident_bytes(int dim, int n, int K, int V, int C, bool mixed) {
 }
 
 // Bands of the resident solve on a mesh of n cells per side with K multigrid
-// levels (1: Jacobi), or 0 where it does not run: one per 512 interior nodes,
-// at most a portable cluster, where a band of every vector fits a CTA's
-// shared memory. 3D FP64 stops at 16^3 cells (Jacobi: 32^3): there the
-// element-sum z-march does half the FP64 operations per node. Jacobi, whose
-// hundreds of iterations are one stencil and two sums each, goes on to 16: one
-// sample of 100^2 3.86 -> 2.93 ms, 20 samples 5.49 -> 4.64 (100 samples, two
-// bands a CTA, 14.2 -> 14.8). With multigrid the second band of a CTA cost the
-// large batches of 32^3 5%, so it stays at 8.
+// levels (1: Jacobi), or 0 where it does not run: one per 512 interior nodes, at
+// most a portable cluster, where a band of every vector fits a CTA's shared
+// memory. Jacobi, whose hundreds of iterations are one stencil and two sums
+// each, goes on to 16 (one sample of 100^2 3.86 -> 2.93 ms, 20 samples 5.49 ->
+// 4.7); with multigrid the second band of a CTA cost large batches 5%. Since the
+// rule cannot look at the batch, a mesh is left to the separate kernels where
+// large batches lose to them: 3D FP64 above 16^3 (Jacobi: 24^3; their z-march
+// does half the FP64 operations per node), 3D mixed multigrid above 16^3 (32^3,
+// 200 samples: 8.4 ms here, 4.9 there), FP64 Jacobi where RES_PER_SM CTAs do not
+// fit an SM (200^2, 100 samples: 142 and 108 ms; 130^2: 34 and 51).
 int resident_bands(int dim, int n, int K, bool mixed) {
   if (n < 2 || K < 1 || K > RES_MAX_LEVELS) return 0;
-  if (n > (dim == 2 ? 256 : mixed ? 40 : K > 1 ? 16 : 32)) return 0;
+  if (n > (dim == 2 ? (K > 1 ? 128 : 256) : K > 1 ? 16 : mixed ? 32 : 24)) return 0;
   const int64_t in = ipow(n - 1, dim);
   int V = 1;
   while (V < RES_PORTABLE && in > (int64_t)V * RES_BAND && 2 * V <= n) V *= 2;
-  if (resident_bytes(dim, n, K, V, V, mixed) > RES_SMEM_MAX) return 0;
-  const bool more = K == 1 && V == RES_PORTABLE && in > (int64_t)V * RES_BAND && RES_MAX_V <= n &&
-                    resident_bytes(dim, n, K, RES_MAX_V, RES_PORTABLE, mixed) <= RES_SMEM_MAX;
-  return more ? RES_MAX_V : V;
+  if (K == 1 && V == RES_PORTABLE && in > (int64_t)V * RES_BAND && RES_MAX_V <= n) V = RES_MAX_V;
+  return resident_bytes(dim, n, K, V, V, mixed) <= (K == 1 && !mixed ? RES_SMEM_SHARE : RES_SMEM_MAX) ? V : 0;
 }
 
 // CTAs per sample for a batch: one per band while the batch leaves room on the
@@ -904,9 +907,7 @@ int resident_bands(int dim, int n, int K, bool mixed) {
 // bands in turn, in the same order of sums).
 static int resident_ctas(int dim, int n, int K, int V, bool mixed, int64_t B, int64_t slots) {
   int C = V;
-  while (C > 1 && B * C > slots &&
-         (C > RES_PORTABLE || resident_bytes(dim, n, K, V, C / 2, mixed) <= RES_SMEM_SHARE))
-    C /= 2;
+  while (C > 1 && B * C > slots && resident_bytes(dim, n, K, V, C / 2, mixed) <= RES_SMEM_SHARE) C /= 2;
   return C;
 }
 

@@ -45,16 +45,15 @@ def layout(dim, n, K, V, C, mixed, solve=True):
 
 
 def bands(dim, n, K, mixed):
-    if n < 2 or K > MAX_LEVELS or n > (256 if dim == 2 else 40 if mixed else 16 if K > 1 else 32):
+    top = (128 if K > 1 else 256) if dim == 2 else 16 if K > 1 else 32 if mixed else 24
+    if n < 2 or K > MAX_LEVELS or n > top:
         return 0
     V = 1
     while V < PORTABLE and (n - 1) ** dim > V * BAND and 2 * V <= n:
         V *= 2
-    if layout(dim, n, K, V, V, mixed)[2] > SMEM:
-        return 0
-    more = K == 1 and V == PORTABLE and (n - 1) ** dim > V * BAND and n >= MAX_V and \
-        layout(dim, n, K, MAX_V, PORTABLE, mixed)[2] <= SMEM
-    return MAX_V if more else V
+    if K == 1 and V == PORTABLE and (n - 1) ** dim > V * BAND and n >= MAX_V:
+        V = MAX_V
+    return V if layout(dim, n, K, V, V, mixed)[2] <= (SHARE if K == 1 and not mixed else SMEM) else 0
 
 
 def band(lv, nd, C, l, rank):
@@ -78,13 +77,13 @@ CASES = [(2, 1 << k, k, mx) for k in range(2, 9) for mx in (False, True)] + \
 def test_bands_slabs_and_shared_memory(dim, n, K, mixed):
     V = bands(dim, n, K, mixed)
     if V == 0:
-        assert n > 32 or (dim == 3 and n > 16 and not mixed)
+        assert n > 128 or (dim == 3 and n > 16)
         return
     C = V
     while C >= 1:
         check(dim, n, K, mixed, V, C)
         C //= 2
-        if C and C < PORTABLE and layout(dim, n, K, V, C, mixed)[2] > SHARE:
+        if C and layout(dim, n, K, V, C, mixed)[2] > SHARE:
             break
 
 
