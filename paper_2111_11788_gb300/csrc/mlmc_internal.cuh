@@ -397,6 +397,7 @@ struct ResidentSolve {
   const double* uc;                   // nested guess on the next coarser mesh (node stride ucs), or null
   int64_t ucs;
   double* u;
+  double* r;                          // mixed form: the FP64 residual, else null
   double* q;
   int32_t *iters, *iters2;            // iters2 may be null
   int box, L, H;

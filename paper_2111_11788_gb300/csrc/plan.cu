@@ -1146,6 +1146,7 @@ mlmc_status resident_mixed(mlmc_plan p, const MeshInfo& mi, MixedWs& w, int64_t 
   r.outer_max = c.outer_max_iter;
   r.scale0 = b_norm(c, mi.g[0]);
   r.u = w.u;
+  r.r = w.r;
   r.iters = w.outer.iters;
   return run_resident(p, r, B);
 }

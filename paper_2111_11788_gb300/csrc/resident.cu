@@ -82,6 +82,7 @@ struct ResArgs {
   const double* uc;    // nested guess: the coarse-mesh solution, or null
   int64_t ucs;
   double* u;           // solution (node arrays of the level-0 stride)
+  double* r;           // mixed: the FP64 residual
   double* q;
   int32_t *iters, *iters2;
   int box, L, H;
@@ -574,15 +575,15 @@ struct Res {
     for (int k = tid; k < cnt * S; k += RES_THREADS) u[z0 * S + k] = x[k];
     finish([&](int js, int o) { return x[js * S + o]; }, it);
   }
-  // Mixed form: FP64 refinement around the FP32 PCG. The solution stays in
-  // global memory (it is touched once per refinement step, and shared memory
-  // is what limits the CTAs on an SM); the FP64 residual goes into the inner
-  // right-hand side as it is formed, scaled by the step before's norm, and is
-  // brought to unit norm once its own is known.
+  // Mixed form: FP64 refinement around the FP32 PCG. The solution and the
+  // residual stay in global memory (they are touched once per refinement step,
+  // and shared memory is what limits the CTAs on an SM); the residual is kept in
+  // FP64 and rounded once, scaled to unit norm, into the inner right-hand side.
   __device__ void solve_mixed() {
     const ResLevel<T>& L = a.lv[0];
     const int n = L.n, S = L.S, z0 = first(0);
     double* u = zero_solution();
+    double* res = a.r + smp * L.ns;
     T* x = at<T>(a.ox);
     T* b = at<T>(L.ob);
     ResScalars& sc = *at<ResScalars>(a.osc);
@@ -594,13 +595,12 @@ struct Res {
     // r = b - A u; stop: 1 converged (or stalled at the rounding floor of the
     // FP64 residual), 2 ended without
     auto step = [&](int outer) {
-      const double inv = 1.0 / scale;
       double dot = 0.0;
       nodes0([&](int js, int o, int i, int j) {
         const double* v0 = u + (z0 + js) * S;
         const double r = resid<double>(n, L.ns, h / 3.0, h / 12.0, kap, coef, v0 - S, v0, v0 + S, z0 + js, o, i, j,
                                        a.bval);
-        b[js * S + o] = (T)(r * inv);
+        res[(z0 + js) * S + o] = r;
         dot = fma(r, r, dot);
       }, [&](int v) {
         part(0, v, dot);
@@ -612,28 +612,27 @@ struct Res {
                       ? 1
                       : (outer >= a.outer_max || !(rho == rho) ? 2 : 0);
         sc.rho = rho;
-        sc.inv = scale / rho;
+        sc.inv = 1.0 / rho;
       });
       scale = sc.rho;
       if (sc.stop == 1) iters = count;
       return sc.stop != 0;
     };
     bool done = false;
-    T unit = T(1);
+    double inv = 1.0 / scale;
     if (a.uc) {
       __syncthreads();   // the zeros of this CTA's slabs before its values
       initial([&](int js, int o, double v) { u[(z0 + js) * S + o] = v; });
       all_sync();
       done = step(0);
-      unit = (T)sc.inv;
+      inv = sc.inv;
     } else {
-      const T b0 = (T)(a.bval / scale);
-      nodes(0, [&](int js, int o, int, int) { b[js * S + o] = b0; });
+      nodes(0, [&](int js, int o, int, int) { res[(z0 + js) * S + o] = a.bval; });
     }
     for (int outer = 1; !done; ++outer) {
       nodes(0, [&](int js, int o, int, int) {
         const int k = js * S + o;
-        b[k] *= unit;
+        b[k] = (T)(res[(z0 + js) * S + o] * inv);
         x[k] = T(0);
       });
       const int it = pcg(a.inner_rtol, a.max_iter);
@@ -644,7 +643,7 @@ struct Res {
       });
       all_sync();
       done = step(outer);
-      unit = (T)sc.inv;
+      inv = sc.inv;
     }
     finish([&](int js, int o) { return u[(z0 + js) * S + o]; }, iters);
   }
@@ -1010,6 +1009,7 @@ cudaError_t launch_resident(cudaStream_t s, const ResidentSolve<T>& r, int64_t B
   a.uc = r.uc;
   a.ucs = r.ucs;
   a.u = r.u;
+  a.r = r.r;
   a.q = r.q;
   a.iters = r.iters;
   a.iters2 = r.iters2;

@@ -5,6 +5,8 @@ largest meshes it takes and the first ones it leaves to the separate kernels.
 
 Tolerances: the solve stops at ||r|| <= 1e-11 ||b||, so Q is within 1e-9 and u
 within 1e-7 of the oracle's direct solution (the bounds of the other solves)."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 
@@ -143,3 +145,23 @@ def test_coupled_batches_repeat_bitwise(m, dim, solver, n0, count, precision):
         for _ in range(8):
             qf, qc, _ = plan.sample_level(1, 0, count)
             assert np.array_equal(qf, want[0]) and np.array_equal(qc, want[1])
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_mixed_residual_is_rounded_once(m, dim):
+    """One unknown, an FP32 operator that inverts exactly (4 in 2D, 2 in 3D) and an FP64 one off it by less than half
+    an FP32 unit: the second refinement step's right-hand side r / ||r|| is then -1 in FP32, and it removes the whole
+    FP64 residual of the first. The operator's entry, the residual and the solution round to 2^-53 each; a residual
+    rounded to FP32 before it is scaled misses by a further 2^-24 of the correction (2e-15 of u)
+    on some of the samples."""
+    count, b, d = 256, 0.5 ** dim, 4.0 if dim == 2 else 2.0
+    eps = 3e-8 + np.arange(count) * 3.5e-11
+    kap = np.repeat(1.5 * (1.0 + eps)[:, None], 2 ** dim, axis=1)
+    assert np.all(kap.astype(np.float32) == np.float32(1.5))
+    st, u, _, it = solve(m, dim, 2, "jacobi", "mixed", kap, outer_max_iter=2)
+    assert st == 0 and np.all(it == 2)
+    D = [Fraction(d) * Fraction(k) / Fraction(3, 2) for k in kap[:, 0]]
+    u1 = Fraction(b) / Fraction(d)
+    want = np.array([float(u1 + (Fraction(b) - x * u1) / Fraction(d)) for x in D])
+    got = u.reshape([count] + [3] * dim)[(slice(None),) + (1,) * dim]
+    assert np.max(np.abs(got - want) / want) <= 5 * 2.0 ** -53
