@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "mlmc_internal.cuh"
+#include "round_share.h"
 
 namespace mlmc {
 
@@ -1496,8 +1497,9 @@ mlmc_status round_launch(mlmc_plan p, const std::vector<int64_t>& first,
     st = build_graph(p, [&]() -> mlmc_status {
       cudaStream_t origin = p->stream;
       const size_t nc = chunks.size();
-      for (const auto& ch : chunks)
-        if (!resident(p->meshes[ch.level], mixed)) p->resident_slots = RESIDENT_SHARED_CTAS;
+      bool larger = false;
+      for (const auto& ch : chunks) larger = larger || !resident(p->meshes[ch.level], mixed);
+      const ScopedLimit share(p->resident_slots, larger ? RESIDENT_SHARED_CTAS : 0);
       cudaEvent_t fork = p->branch_ev[0];
       CK(cudaEventRecord(fork, origin));
       // chunks finest level first, each on its own branch
@@ -1515,7 +1517,6 @@ mlmc_status round_launch(mlmc_plan p, const std::vector<int64_t>& first,
         p->stream = origin;
         if (s2 == MLMC_OK) CK(cudaEventRecord(p->branch_ev[1 + order[i]], S));
       }
-      p->resident_slots = 0;
       // each level's chunks are folded in sample order on the branch of its first chunk
       for (int l = 0; l < L1 && s2 == MLMC_OK; ++l) {
         int head = -1;
@@ -1659,8 +1660,9 @@ mlmc_status group_launch(mlmc_plan p, const std::vector<int64_t>& first, char* w
     CK(cudaEventRecord(p->branch_ev[0], origin));
     int nb = 0;
     mlmc_status s2 = MLMC_OK;
-    for (int l = 0; l < L1; ++l)
-      if (B[l] > 0 && !resident(p->meshes[l], mixed)) p->resident_slots = RESIDENT_SHARED_CTAS;
+    bool larger = false;
+    for (int l = 0; l < L1; ++l) larger = larger || (B[l] > 0 && !resident(p->meshes[l], mixed));
+    const ScopedLimit share(p->resident_slots, larger ? RESIDENT_SHARED_CTAS : 0);
     for (int l = L1 - 1; l >= 0 && s2 == MLMC_OK; --l) {
       if (B[l] <= 0) continue;
       cudaStream_t S = p->branch[nb];
@@ -1671,7 +1673,6 @@ mlmc_status group_launch(mlmc_plan p, const std::vector<int64_t>& first, char* w
       if (s2 == MLMC_OK) CK(cudaEventRecord(p->branch_ev[1 + nb], S));
       ++nb;
     }
-    p->resident_slots = 0;
     for (int i = 0; i < nb && s2 == MLMC_OK; ++i) CK(cudaStreamWaitEvent(origin, p->branch_ev[1 + i], 0));
     return s2;
   }, &rec);
