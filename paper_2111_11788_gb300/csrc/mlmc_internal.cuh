@@ -403,12 +403,6 @@ struct ResidentSolve {
   int box, L, H;
   double inv_vol;
 };
-// CTAs a resident solve may take in a round that also solves larger meshes: it
-// holds all its CTAs' registers while it waits on barriers, and the larger
-// meshes' kernels, which fill the HBM or the FP64 pipe, run beside it (a mixed
-// 2D run of 32^2 .. 512^2: 21.1 ms with no limit, 20.5 with 304 CTAs, 19.9 with
-// 152, 19.7 with 114, 20.4 with 76, 25.9 with 38).
-constexpr int64_t RESIDENT_SHARED_CTAS = 114;
 // 0 where the resident solve does not run (a function of mesh and form alone)
 int resident_bands(int dim, int n, int K, bool mixed);
 template <class T>

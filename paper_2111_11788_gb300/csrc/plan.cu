@@ -1088,6 +1088,17 @@ bool resident(const MeshInfo& mi, bool mixed) {
   return mi.K <= MAX_RESIDENT_LEVELS && resident_bands(mi.g[0].dim, mi.n, mi.K, mixed) > 0;
 }
 
+// The solves of `count` coupled samples of a level.
+void add_level_work(mlmc_plan p, int level, int64_t count, RoundWork& w) {
+  const bool mixed = is_mixed(p);
+  auto on = [&](int m) {
+    const MeshInfo& mi = p->meshes[m];
+    return RoundWork::of(mi.g[0].dim, mi.n, mi.K == 1, count);
+  };
+  w.add_level(on(level), resident(p->meshes[level], mixed), level > 0 ? on(level - 1) : 0.0,
+              level > 0 && resident(p->meshes[level - 1], mixed));
+}
+
 template <class T>
 ResidentSolve<T> resident_args(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, double* q_dev, int32_t* iters_dev,
                                const Guess& gs) {
@@ -1497,9 +1508,9 @@ mlmc_status round_launch(mlmc_plan p, const std::vector<int64_t>& first,
     st = build_graph(p, [&]() -> mlmc_status {
       cudaStream_t origin = p->stream;
       const size_t nc = chunks.size();
-      bool larger = false;
-      for (const auto& ch : chunks) larger = larger || !resident(p->meshes[ch.level], mixed);
-      const ScopedLimit share(p->resident_slots, larger ? RESIDENT_SHARED_CTAS : 0);
+      RoundWork work;
+      for (const auto& ch : chunks) add_level_work(p, ch.level, ch.count, work);
+      const ScopedLimit share(p->resident_slots, resident_limit(work, mixed));
       cudaEvent_t fork = p->branch_ev[0];
       CK(cudaEventRecord(fork, origin));
       // chunks finest level first, each on its own branch
@@ -1660,9 +1671,9 @@ mlmc_status group_launch(mlmc_plan p, const std::vector<int64_t>& first, char* w
     CK(cudaEventRecord(p->branch_ev[0], origin));
     int nb = 0;
     mlmc_status s2 = MLMC_OK;
-    bool larger = false;
-    for (int l = 0; l < L1; ++l) larger = larger || (B[l] > 0 && !resident(p->meshes[l], mixed));
-    const ScopedLimit share(p->resident_slots, larger ? RESIDENT_SHARED_CTAS : 0);
+    RoundWork work;
+    for (int l = 0; l < L1; ++l) add_level_work(p, l, B[l], work);
+    const ScopedLimit share(p->resident_slots, resident_limit(work, mixed));
     for (int l = L1 - 1; l >= 0 && s2 == MLMC_OK; --l) {
       if (B[l] <= 0) continue;
       cudaStream_t S = p->branch[nb];
