@@ -880,25 +880,38 @@ static size_t resident_bytes(int dim, int n, int K, int V, int C, bool mixed) {
   return mixed ? resident_layout(dim, n, K, V, C, f) : resident_layout(dim, n, K, V, C, d);
 }
 
+// Largest mesh (cells per side) whose solves run resident. The rule looks at the
+// mesh alone, so that a sample's bits do not depend on its batch, and takes a
+// mesh where 100 samples are no slower than on the separate kernels (one sample
+// is 1.7 to 4 times as fast). ms resident / separate kernels:
+//   2D FP64 GMG 128^2: 1 sample 0.68/1.19, 100 2.8/3.6, 256 7.0/7.2, 400 10.7/9.7, 1000 25.8/21.6
+//   2D mixed GMG 128^2: 1 0.56/0.96, 100 1.3/1.9, 400 3.9/4.2, 1000 9.1/8.6
+//   2D FP64 GMG 64^2: 1000 6.5/7.2, 4000 24.9/23.6; mixed: 4000 9.9/9.8
+//   3D GMG 16^3: FP64 1000 12.4/15.6, mixed 3000 10.5/15.3; 32^3 mixed: 200 8.4/4.9
+//   2D FP64 Jacobi: 150^2 100 50.5/60.4, 300 140/129; 170^2 100 79.2/82.5, 300 234/182; 179^2 100 91.4/89.7
+//   2D mixed Jacobi: 200^2 300 147/155, 256^2 100 134/144, 300 372/333
+//   3D FP64 Jacobi 24^3: 300 33.0/33.5; 32^3: 64 29.6/18.5
+//   3D mixed Jacobi: 30^3 100 6.8/9.5, 300 19.9/20.8; 31^3 100 11.5/10.0, 32^3 12.3/9.8
+// So on the largest meshes batches of several hundred samples and more take
+// longer than they would on the separate kernels, up to 30%.
+static int resident_cells(int dim, int K, bool mixed) {
+  if (K > 1) return dim == 2 ? 128 : 16;
+  return dim == 2 ? (mixed ? 256 : 170) : (mixed ? 30 : 24);
+}
+
 // Bands of the resident solve on a mesh of n cells per side with K multigrid
 // levels (1: Jacobi), or 0 where it does not run: one per 512 interior nodes, at
-// most a portable cluster, where a band of every vector fits a CTA's shared
-// memory. Jacobi, whose hundreds of iterations are one stencil and two sums
-// each, goes on to 16 (one sample of 100^2 3.86 -> 2.93 ms, 20 samples 5.49 ->
-// 4.7); with multigrid the second band of a CTA cost large batches 5%. Since the
-// rule cannot look at the batch, a mesh is left to the separate kernels where
-// large batches lose to them: 3D FP64 above 16^3 (Jacobi: 24^3; their z-march
-// does half the FP64 operations per node), 3D mixed multigrid above 16^3 (32^3,
-// 200 samples: 8.4 ms here, 4.9 there), FP64 Jacobi where RES_PER_SM CTAs do not
-// fit an SM (200^2, 100 samples: 142 and 108 ms; 130^2: 34 and 51).
+// most a portable cluster. Jacobi, whose hundreds of iterations are one stencil
+// and two sums each, goes on to 16 (one sample of 100^2 3.86 -> 2.93 ms, 20
+// samples 5.49 -> 4.7); with multigrid the second band of a CTA cost large
+// batches 5%.
 int resident_bands(int dim, int n, int K, bool mixed) {
-  if (n < 2 || K < 1 || K > RES_MAX_LEVELS) return 0;
-  if (n > (dim == 2 ? (K > 1 ? 128 : 256) : K > 1 ? 16 : mixed ? 32 : 24)) return 0;
+  if (n < 2 || K < 1 || K > RES_MAX_LEVELS || n > resident_cells(dim, K, mixed)) return 0;
   const int64_t in = ipow(n - 1, dim);
   int V = 1;
   while (V < RES_PORTABLE && in > (int64_t)V * RES_BAND && 2 * V <= n) V *= 2;
   if (K == 1 && V == RES_PORTABLE && in > (int64_t)V * RES_BAND && RES_MAX_V <= n) V = RES_MAX_V;
-  return resident_bytes(dim, n, K, V, V, mixed) <= (K == 1 && !mixed ? RES_SMEM_SHARE : RES_SMEM_MAX) ? V : 0;
+  return resident_bytes(dim, n, K, V, V, mixed) <= RES_SMEM_MAX ? V : 0;
 }
 
 // CTAs per sample for a batch: one per band while the batch leaves room on the

@@ -71,6 +71,25 @@ def test_solve_matches_oracle(m, dim, solver, n, precision):
             assert not full.take([0, n], axis=a).any()
 
 
+@pytest.mark.parametrize("dim,solver,precision,last,first_left", [
+    (2, "gmg", "fp64", 128, 256), (2, "gmg", "mixed", 128, 256), (3, "gmg", "fp64", 16, 32), (3, "gmg", "mixed", 16, 32),
+    (2, "jacobi", "fp64", 170, 171), (2, "jacobi", "mixed", 256, 257), (3, "jacobi", "fp64", 24, 25),
+    (3, "jacobi", "mixed", 30, 31)])
+def test_the_meshes_that_run_resident(m, dim, solver, precision, last, first_left):
+    """By the launches of a solve: two of setup and the solve, against hundreds of the separate kernels. The meshes
+    beyond `last` are those where 100 samples are faster on the separate kernels."""
+    for n, resident in ((last, True), (first_left, False)):
+        cfg = m.config(dim=dim, n_levels=1, coarse_cells=n, solver=solver, precision=precision, rtol=1e-8)
+        k = torch.ones(m.elem_stride(dim, n), dtype=torch.float64, device="cuda")
+        u = torch.zeros(m.node_stride(dim, n), dtype=torch.float64, device="cuda")
+        q = torch.zeros(1, dtype=torch.float64, device="cuda")
+        with m.Plan(cfg, stream()) as plan:
+            before = plan.launch_count()
+            plan.solve(0, k.data_ptr(), 1, u.data_ptr(), q.data_ptr(), 0)
+            torch.cuda.synchronize()
+            assert (plan.launch_count() - before <= 3) == resident, n
+
+
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("dim,solver,n", [(2, "gmg", 64), (2, "jacobi", 45), (3, "gmg", 16), (2, "gmg", 8)])
 def test_results_do_not_depend_on_the_batch(m, dim, solver, n, precision):

@@ -44,16 +44,22 @@ def layout(dim, n, K, V, C, mixed, solve=True):
     return lv, nd, (off + 15) // 16 * 16
 
 
+def cells(dim, K, mixed):
+    """Largest mesh whose solves run resident."""
+    if K > 1:
+        return 128 if dim == 2 else 16
+    return (256 if mixed else 170) if dim == 2 else (30 if mixed else 24)
+
+
 def bands(dim, n, K, mixed):
-    top = (128 if K > 1 else 256) if dim == 2 else 16 if K > 1 else 32 if mixed else 24
-    if n < 2 or K > MAX_LEVELS or n > top:
+    if n < 2 or K > MAX_LEVELS or n > cells(dim, K, mixed):
         return 0
     V = 1
     while V < PORTABLE and (n - 1) ** dim > V * BAND and 2 * V <= n:
         V *= 2
     if K == 1 and V == PORTABLE and (n - 1) ** dim > V * BAND and n >= MAX_V:
         V = MAX_V
-    return V if layout(dim, n, K, V, V, mixed)[2] <= (SHARE if K == 1 and not mixed else SMEM) else 0
+    return V if layout(dim, n, K, V, V, mixed)[2] <= SMEM else 0
 
 
 def band(lv, nd, C, l, rank):
@@ -69,15 +75,16 @@ def band(lv, nd, C, l, rank):
 
 CASES = [(2, 1 << k, k, mx) for k in range(2, 9) for mx in (False, True)] + \
         [(3, 1 << k, k, mx) for k in range(2, 7) for mx in (False, True)] + \
-        [(2, n, 1, mx) for n in (2, 3, 9, 31, 45, 100, 129, 200, 235, 256) for mx in (False, True)] + \
-        [(3, n, 1, mx) for n in (2, 3, 9, 17, 25, 31, 32, 40) for mx in (False, True)]
+        [(2, n, 1, mx) for n in (2, 3, 9, 31, 45, 67, 100, 129, 170, 171, 200, 235, 256, 257) for mx in (False, True)] + \
+        [(3, n, 1, mx) for n in (2, 3, 9, 17, 24, 25, 30, 31, 40) for mx in (False, True)]
 
 
 @pytest.mark.parametrize("dim,n,K,mixed", CASES)
 def test_bands_slabs_and_shared_memory(dim, n, K, mixed):
     V = bands(dim, n, K, mixed)
+    # every mesh up to the largest has its bands: none is left out by its shared memory
+    assert (V > 0) == (n <= cells(dim, K, mixed))
     if V == 0:
-        assert n > 128 or (dim == 3 and n > 16)
         return
     C = V
     while C >= 1:
