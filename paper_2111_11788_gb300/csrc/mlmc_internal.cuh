@@ -284,6 +284,9 @@ cudaError_t resid64(cudaStream_t s, const Grid& g, const double* kappa, const do
 // sample stride 4 ns) for the FP64 element-sum z-march.
 cudaError_t ksum(cudaStream_t s, const Grid& g, const double* kappa, double* ks, int64_t B, double omega = 0.0,
                  double* w = nullptr);
+// whether the FP32 post-smoother of this grid is one kernel, which forms e = W b
+// itself: mg_pre does not store it and both take null
+bool post32_is_fused(const Grid& g);
 // nested initial guess: x = P uc (trilinear interpolation from grid `coarse`)
 cudaError_t prolong_guess(cudaStream_t s, const Grid& g, const Grid& coarse, const double* uc,
                           double* x, const int32_t* active, int64_t B, Prof p);

@@ -100,14 +100,36 @@ struct SolveWs {
   int32_t* execs;    // device count of loop-body executions (graph-driven loop)
 };
 
+// Whether the solves on this mesh run as one resident launch (resident.cu).
+bool resident(const MeshInfo& mi, bool mixed) {
+  return mi.K <= MAX_RESIDENT_LEVELS && resident_bands(mi.g[0].dim, mi.n, mi.K, mixed) > 0;
+}
+
+// The first of the levels below the finest whose grids have at most BOTTOM_MAX_N2
+// (2D) or BOTTOM_MAX_N3 (3D) cells per side: they run as one fused kernel, a
+// cluster of CTAs per sample (resident.cu, k_bottom). K - 1 where there are not
+// two of them.
+int bottom_level(const MeshInfo& mi) {
+  const int K = mi.K, nmax = mi.g[0].dim == 2 ? BOTTOM_MAX_N2 : BOTTOM_MAX_N3;
+  int k0 = K - 1;
+  while (k0 - 1 >= 1 && mi.g[k0 - 1].n <= nmax) --k0;
+  return K - k0 <= MAX_BOTTOM ? k0 : K - 1;
+}
+
+// Takes the arrays that the separate kernels touch: k_bottom keeps its levels'
+// vectors in shared memory, and the FP32 smoothers form e = W b again (3D: where
+// the post-smoother is one kernel). A resident solve uses only kappa, the weights,
+// the 2D coefficients and x; the rest is reserved for its mesh all the same.
 template <class T>
 void carve_solve(Carve& c, const MeshInfo& mi, int64_t B, bool own_kappa0, SolveWs<T>& w) {
   // the FP64 stencils run on precomputed operator data where a stencil
   // kernel runs: 2D coefficients (3 node + 1 element arrays per level), 3D
   // kappa sums (4 node arrays per level)
-  const bool coef = sizeof(T) == 8;
+  const bool f64 = sizeof(T) == 8;
   const bool d2c = mi.g[0].dim == 2;
+  const int kd = bottom_level(mi);   // levels above it are smoothed by kernels of their own
   const Grid& g0 = mi.g[0];
+  auto node = [&](bool used, const Grid& g) { return used ? c.take<T>(B * g.ns) : nullptr; };
   w.x = c.take<T>(B * g0.ns);
   w.r = c.take<T>(B * g0.ns);
   w.p0 = c.take<T>(B * g0.ns);
@@ -116,14 +138,17 @@ void carve_solve(Carve& c, const MeshInfo& mi, int64_t B, bool own_kappa0, Solve
   w.z = c.take<T>(B * g0.ns);
   for (int k = 0; k < mi.K; ++k) {
     const Grid& g = mi.g[k];
+    const bool coef = f64 && (k == 0 || k < mi.K - 1);
     w.kap[k] = (k == 0 && !own_kappa0) ? nullptr : c.take<T>(B * g.es);
-    w.coef[k] = (coef && (k == 0 || k < mi.K - 1)) ? c.take<T>(B * (d2c ? 3 * g.ns + g.es : 4 * g.ns)) : nullptr;
+    w.coef[k] = coef ? c.take<T>(B * (d2c ? 3 * g.ns + g.es : 4 * g.ns)) : nullptr;
     w.w[k] = c.take<T>(B * g.ns);
     if (mi.K > 1) {
-      w.e[k] = c.take<T>(B * g.ns);
-      w.r1[k] = (k < mi.K - 1) ? c.take<T>(B * g.ns) : nullptr;
-      w.bk[k] = (k == 0) ? w.r : c.take<T>(B * g.ns);
-      w.eo[k] = (k == 0) ? w.z : ((k < mi.K - 1) ? c.take<T>(B * g.ns) : w.e[k]);
+      const bool smooth = k < kd;
+      const bool stored = f64 || !(d2c || d3::post32_is_fused(g));   // e
+      w.e[k] = node((smooth && stored) || (k == kd && k == mi.K - 1), g);
+      w.r1[k] = node(smooth, g);
+      w.bk[k] = k == 0 ? w.r : node(k <= kd, g);
+      w.eo[k] = k == 0 ? w.z : (k < mi.K - 1 ? node(k <= kd, g) : w.e[k]);
     }
   }
   w.part = c.take<double>(B * g0.tiles());
@@ -693,22 +718,16 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
     return MLMC_OK;
   }
   const int K = mi.K;
-  // the levels below the finest whose grids have at most BOTTOM_MAX_N2 (2D)
-  // or BOTTOM_MAX_N3 (3D) cells per side run as one fused kernel
-  // (k0 .. K-1), one CTA per sample
-  const int nmax = g0.dim == 2 ? BOTTOM_MAX_N2 : BOTTOM_MAX_N3;
-  int k0 = K - 1;
-  while (k0 - 1 >= 1 && mi.g[k0 - 1].n <= nmax) --k0;
-  const bool fuse = k0 < K - 1 && K - k0 <= MAX_BOTTOM;
-  const int kd = fuse ? k0 : K - 1;   // levels above the bottom
-  // node arrays a smoother moves: FP32 forms e = W b again instead of keeping it (3D: on the four-row tiles)
-  const double na = sizeof(T) == 4 && (g0.dim == 2 || g0.zt == 0) ? 3.0 : 4.0;
+  const int kd = bottom_level(mi);   // levels above the bottom
+  const bool fuse = kd < K - 1;
+  // node arrays a smoother moves: with e, or without where it is formed again
+  auto na = [&](int k) { return w.e[k] ? 4.0 : 3.0; };
   for (int k = 0; k < kd; ++k) {
     const Grid& g = mi.g[k];
     const double nn = nodes_of(g), ne = elems_of(g);
     CK(run(p, KID_MG_PRE, [&] {
       return op::mg_pre<T>(s, g, w.kap[k], w.w[k], w.bk[k], w.e[k], w.r1[k], w.sc.active, B,
-                           prof_for(p, KID_MG_PRE, (na * nn + ne) * vb), w.coef[k]);
+                           prof_for(p, KID_MG_PRE, (na(k) * nn + ne) * vb), w.coef[k]);
     }));
     CK(run(p, KID_RESTRICT, [&] {
       return op::restrict_<T>(s, g, mi.g[k + 1], w.r1[k], w.bk[k + 1], w.sc.active, B,
@@ -717,18 +736,18 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
   }
   if (fuse) {
     BottomLevels<T> lv{};
-    lv.L = K - k0;
+    lv.L = K - kd;
     lv.cycles = g0.dim == 2 && g0.n >= BOTTOM_TWICE_N2 ? 2 : 1;
-    double bytes = 2 * nodes_of(mi.g[k0]);
+    double bytes = 2 * nodes_of(mi.g[kd]);
     for (int l = 0; l < lv.L; ++l) {
-      lv.g[l] = mi.g[k0 + l];
-      lv.kap[l] = w.kap[k0 + l];
-      lv.coef[l] = w.coef[k0 + l];
-      lv.w[l] = w.w[k0 + l];
-      bytes += nodes_of(mi.g[k0 + l]) + elems_of(mi.g[k0 + l]);
+      lv.g[l] = mi.g[kd + l];
+      lv.kap[l] = w.kap[kd + l];
+      lv.coef[l] = w.coef[kd + l];
+      lv.w[l] = w.w[kd + l];
+      bytes += nodes_of(mi.g[kd + l]) + elems_of(mi.g[kd + l]);
     }
     CK(run(p, KID_MG_BOTTOM, [&] {
-      return launch_bottom<T>(s, lv, w.bk[k0], w.eo[k0], w.sc.active, B,
+      return launch_bottom<T>(s, lv, w.bk[kd], w.eo[kd], w.sc.active, B,
                               prof_for(p, KID_MG_BOTTOM, bytes * vb));
     }));
   } else {
@@ -743,7 +762,7 @@ mlmc_status precondition(mlmc_plan p, const MeshInfo& mi, SolveWs<T>& w, int64_t
       // r1[k] is dead once restricted: it serves as the 3D scratch for e + P e_c
       return op::mg_post<T>(s, g, mi.g[k + 1], w.kap[k], w.w[k], w.bk[k], w.e[k], w.eo[k + 1],
                             w.eo[k], w.r1[k], w.sc.active, k == 0 ? w.part : nullptr, B,
-                            prof_for(p, KID_MG_POST, (na * nn + ne + nc) * vb), w.coef[k]);
+                            prof_for(p, KID_MG_POST, (na(k) * nn + ne + nc) * vb), w.coef[k]);
     }));
   }
   *tiles = g0.tiles_s;
@@ -1081,11 +1100,6 @@ mlmc_status fp64_epilogue(mlmc_plan p, const MeshInfo& mi, SolveWs<double>& w, i
   if (st != MLMC_OK) return st;
   if (iters_dev) CK(cudaMemcpyAsync(iters_dev, w.sc.iters, sizeof(int32_t) * B, cudaMemcpyDeviceToDevice, p->stream));
   return MLMC_OK;
-}
-
-// Whether the solves on this mesh run as one resident launch (resident.cu).
-bool resident(const MeshInfo& mi, bool mixed) {
-  return mi.K <= MAX_RESIDENT_LEVELS && resident_bands(mi.g[0].dim, mi.n, mi.K, mixed) > 0;
 }
 
 // The solves of `count` coupled samples of a level.

@@ -2058,6 +2058,8 @@ inline dim3 block3() { return dim3(BX, BY, 1); }
 
 namespace d3 {
 
+bool post32_is_fused(const Grid& g) { return zm_wide(g) && g.zt == 0; }
+
 template <class T>
 cudaError_t apply(cudaStream_t s, const Grid& g, const T* kappa, const T* x, T* y, int64_t B, Prof p) {
   launch_zm3<T>(s, flat_chunks<T>(g, B), B, kappa, LdX<T>{x, g.ns}, nullptr, EpiApply<T>{y, g.ns}, nullptr, p);
@@ -2085,10 +2087,7 @@ cudaError_t pcg_pq(cudaStream_t s, const Grid& g, const T* kappa, const T* z, co
 template <class T>
 cudaError_t mg_pre(cudaStream_t s, const Grid& g, const T* kappa, const T* w, const T* b, T* e, T* r1,
                    const int32_t* active, int64_t B, Prof p, const T* ks) {
-  // FP32 levels whose post-smoother forms e = W b again do not store it (mg_post's test)
-  const bool keep = !(sizeof(T) == 4 && zm_wide(g) && g.zt == 0 &&
-                      (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) == 0);
-  launch_zm3<T>(s, flat_chunks<T>(g, B), B, kappa, LdWb<T>{w, b, g.ns}, active, EpiMgRes<T>{b, r1, keep ? e : nullptr, g.ns}, nullptr, p,
+  launch_zm3<T>(s, flat_chunks<T>(g, B), B, kappa, LdWb<T>{w, b, g.ns}, active, EpiMgRes<T>{b, r1, e, g.ns}, nullptr, p,
                 ks);
   return cudaGetLastError();
 }
@@ -2112,8 +2111,10 @@ cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* 
                     double* part, int64_t B, Prof p, const T* ks) {
   const Grid h = part ? g : flat_chunks<T>(g, B);
   if constexpr (std::is_same<T, float>::value) {
-    // one kernel (the arrays are a plan's, 256-byte aligned; e is not read)
-    if (zm_wide(g) && g.zt == 0 && (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) == 0) {
+    // one kernel, which forms e itself (the arrays are a plan's, 256-byte aligned)
+    if (!e) {
+      if (!post32_is_fused(g) || (((uintptr_t)w | (uintptr_t)b | (uintptr_t)kappa) & 15) != 0)
+        return cudaErrorInvalidValue;
       launch_zm3n(s, h, B, kappa, LdPostf{w, b, ec, g.ns, coarse.ns}, active, EpiMgPost<float>{w, b, out, g.ns}, part,
                   p);
       return cudaGetLastError();

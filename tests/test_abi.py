@@ -194,3 +194,39 @@ def test_coef_count_matches_the_oracle_mode_sets(m):
         cfg = m.config(dim=dim, modes_per_dim=mpd, total_order=order)
         assert m.coef_count(cfg) == kle.n_modes(dim, mpd, None if order < 0 else order)
     assert m.lib().mlmc_coef_count(ctypes.byref(m.config(dim=4))) == -1
+
+
+def per_sample_bytes(m, dim, n, solver, precision):
+    """Workspace bytes that one more sample of a level without a coarse partner takes."""
+    cfg = m.config(dim=dim, n_levels=1, coarse_cells=n, solver=solver, precision=precision, modes_per_dim=1)
+    size = lambda B: m.lib().mlmc_round_bytes(ctypes.byref(cfg), (ctypes.c_int64 * 1)(B))
+    return (size(3000) - size(1000)) / 2000
+
+
+@pytest.mark.parametrize("dim,n,precision", [(2, 512, "mixed"), (2, 1024, "fp64"), (3, 64, "mixed"), (3, 128, "fp64")])
+def test_round_bytes_hold_what_the_kernels_touch(m, dim, n, precision):
+    """Multigrid on separate kernels: vectors of the levels below the fused ones, and the e that the FP32 smoothers form
+    again, take no memory."""
+    ns, es = (lambda k: m.node_stride(dim, n >> k)), (lambda k: m.elem_stride(dim, n >> k))
+    K, f64 = n.bit_length() - 1, precision == "fp64"
+    top = n.bit_length() - (7 if dim == 2 else 5)             # levels above those of 64^2 (16^3) cells
+    words = sum(es(k) + ns(k) for k in range(K))              # kappa and smoother weights
+    words += 6 * ns(0) + sum(ns(k) for k in range(top)) + 2 * sum(ns(k) for k in range(1, top + 1))
+    doubles = 0
+    if f64:   # e and operator data
+        words += sum(ns(k) for k in range(top)) + sum(3 * ns(k) + es(k) if dim == 2 else 4 * ns(k) for k in range(K - 1))
+    else:     # u, r, kappa, operator data
+        doubles = 2 * ns(0) + es(0) + (3 * ns(0) + es(0) if dim == 2 else 4 * ns(0))
+    want = words * (8 if f64 else 4) + doubles * 8
+    got = per_sample_bytes(m, dim, n, "gmg", precision)
+    # and the partial sums, the coefficients of the field, results and scalars
+    assert want <= got <= want * 1.002 + 1024, (got, want)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("dim,solver,sizes", [(2, "gmg", [1 << k for k in range(1, 12)]),
+                                              (3, "gmg", [1 << k for k in range(1, 10)])])
+def test_the_coarse_solve_fits_the_fine_ones_region(m, dim, solver, precision, sizes):
+    """A coupled batch's region is that of its fine mesh, and its coarse solve runs in it."""
+    bytes_ = [per_sample_bytes(m, dim, n, solver, precision) for n in sizes]
+    assert bytes_ == sorted(bytes_)
