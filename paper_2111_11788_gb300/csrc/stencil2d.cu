@@ -535,13 +535,13 @@ __global__ void __launch_bounds__(SBLOCK) k_mgpre2(Grid g, const T* __restrict__
   const Strip s = strip_of<SR>(g);
   const T* w_ = W + b * g.ns;
   const T* bv = Bv + b * g.ns;
-  T* e = E + b * g.ns;
   T* r1 = R1 + b * g.ns;
   auto field = [&](int c, int j) {
     const int64_t o = (int64_t)j * s.N1 + c;
     return __ldg(w_ + o) * __ldg(bv + o);
   };
   if constexpr (kResidualForm<T>) {
+    T* e = E + b * g.ns;
     stream_strip_r<T, C, true>(s, K + b * cs, g.ns, field,
                                [&](int j) { return __ldg(bv + (int64_t)j * s.N1 + s.c); },
                                [&](int j, T ev, T rv, T) {
@@ -576,38 +576,6 @@ __device__ __forceinline__ T prolong2(const T* __restrict__ Ec, int nc, int i, i
   T v1 = __ldg(e + N1c);
   if (ox) v1 = T(0.5) * (v1 + __ldg(e + N1c + 1));
   return T(0.5) * (v0 + v1);
-}
-
-// The same value split into its loads (the node's e and the coarse values
-// it interpolates, 0 where the parity needs none) and their combination, for
-// fields formed one row after they are fetched.
-template <class T>
-struct RawP2 {
-  T e, a, b, c, d;
-};
-template <class T>
-__device__ __forceinline__ RawP2<T> prolong2_fetch(const T* __restrict__ e_node, const T* __restrict__ Ec,
-                                                   int nc, int i, int j) {
-  const int N1c = nc + 1;
-  const T* p = Ec + (int64_t)(j >> 1) * N1c + (i >> 1);
-  const bool ox = i & 1, oy = j & 1;
-  RawP2<T> r;
-  r.e = __ldg(e_node);
-  r.a = __ldg(p);
-  r.b = ox ? __ldg(p + 1) : T(0);
-  r.c = oy ? __ldg(p + N1c) : T(0);
-  r.d = (ox && oy) ? __ldg(p + N1c + 1) : T(0);
-  return r;
-}
-template <class T>
-__device__ __forceinline__ T prolong2_form(const RawP2<T>& r, int i, int j) {
-  const bool ox = i & 1, oy = j & 1;
-  T v0 = r.a;
-  if (ox) v0 = T(0.5) * (v0 + r.b);
-  if (!oy) return r.e + v0;
-  T v1 = r.c;
-  if (ox) v1 = T(0.5) * (v1 + r.d);
-  return r.e + T(0.5) * (v0 + v1);
 }
 
 // Bilinear prolongation of the coarse correction, streamed down one fine
@@ -648,53 +616,38 @@ struct Prolong2 {
 };
 
 // out = e' + W (b - A e'), e' = e + P ec; partials of b.out when part != nullptr.
-template <class T, bool C, int SR>
-__global__ void __launch_bounds__(SBLOCK) k_mgpost2(Grid g, int64_t nsc, const T* __restrict__ K, int64_t cs,
-                                                    const T* __restrict__ W,
-                                                    const T* __restrict__ Bv,
-                                                    const T* __restrict__ E,
-                                                    const T* __restrict__ Ec, T* __restrict__ Out,
+// The FP64 form (FP32: k_mgpost2f).
+template <bool C, int SR>
+__global__ void __launch_bounds__(SBLOCK) k_mgpost2(Grid g, int64_t nsc, const double* __restrict__ K, int64_t cs,
+                                                    const double* __restrict__ W,
+                                                    const double* __restrict__ Bv,
+                                                    const double* __restrict__ E,
+                                                    const double* __restrict__ Ec, double* __restrict__ Out,
                                                     const int32_t* __restrict__ active,
                                                     double* __restrict__ part, Prof prof) {
   const int64_t b = blockIdx.z;
   if (!active[b]) return;
   const Strip s = strip_of<SR>(g);
   const int nc = g.n / 2;
-  const T* ec = Ec + b * nsc;
-  const T* e = E + b * g.ns;
-  const T* w_ = W + b * g.ns;
-  const T* bv = Bv + b * g.ns;
-  T* out = Out + b * g.ns;
-  T dot = T(0);
-  if constexpr (kResidualForm<T>) {
-    Prolong2<T> pr{ec, nc + 1};
-    stream_strip_r<T, C, true>(s, K + b * cs, g.ns,
-                               [&](int c, int j) { return pr.add(__ldg(e + (int64_t)j * s.N1 + c), c, j); },
-                               [&](int j) { return __ldg(bv + (int64_t)j * s.N1 + s.c); },
-                               [&](int j, T ev, T rv, T bval) {
-                                 const int64_t o = (int64_t)j * s.N1 + s.c;
-                                 T ov = T(0);
-                                 if (interior2(s.n, s.c, j)) {
-                                   ov = fma(__ldg(w_ + o), rv, ev);
-                                   dot = fma(bval, ov, dot);
-                                 }
-                                 out[o] = ov;
-                               });
-  } else {
-    stream_strip_f<T, C>(s, K + b * cs, g.ns,
-                       [&](int c, int j) { return prolong2_fetch(e + (int64_t)j * s.N1 + c, ec, nc, c, j); },
-                       [&](const RawP2<T>& r, int c, int j) { return prolong2_form(r, c, j); },
-                       [&](int j, T ev, T ax) {
-                         const int64_t o = (int64_t)j * s.N1 + s.c;
-                         T ov = T(0);
-                         if (interior2(s.n, s.c, j)) {
-                           const T bval = __ldg(bv + o);
-                           ov = fma(__ldg(w_ + o), bval - ax, ev);
-                           dot = fma(bval, ov, dot);
-                         }
-                         out[o] = ov;
-                       });
-  }
+  const double* ec = Ec + b * nsc;
+  const double* e = E + b * g.ns;
+  const double* w_ = W + b * g.ns;
+  const double* bv = Bv + b * g.ns;
+  double* out = Out + b * g.ns;
+  double dot = 0.0;
+  Prolong2<double> pr{ec, nc + 1};
+  stream_strip_r<double, C, true>(s, K + b * cs, g.ns,
+                                  [&](int c, int j) { return pr.add(__ldg(e + (int64_t)j * s.N1 + c), c, j); },
+                                  [&](int j) { return __ldg(bv + (int64_t)j * s.N1 + s.c); },
+                                  [&](int j, double ev, double rv, double bval) {
+                                    const int64_t o = (int64_t)j * s.N1 + s.c;
+                                    double ov = 0.0;
+                                    if (interior2(s.n, s.c, j)) {
+                                      ov = fma(__ldg(w_ + o), rv, ev);
+                                      dot = fma(bval, ov, dot);
+                                    }
+                                    out[o] = ov;
+                                  });
   if (part) warp_partial(dot, part, s.part_idx);
   prof_tick(prof);
 }
@@ -723,7 +676,7 @@ __global__ void __launch_bounds__(SBLOCK, 9) k_mgpost2f(Grid g, int64_t nsc, con
   // x(2J + 1) = e + H(J)/4 + H(J + 1)/4 and x(2J + 2) = e + H(J + 1)/2, with
   // H(J) the sum of the coarse values at columns c / 2 and (c + 1) / 2 of
   // coarse row J. The fetch of a pair loads coarse row J + 1; H(J) is the
-  // previous pair's (hprev). Bitwise equal to prolong2_form (the scalings
+  // previous pair's (hprev). Bitwise equal to the textbook form (the scalings
   // are exact).
   static_assert(SR % 2 == 0, "strips start on even rows");
   const int n = s.n, c = s.c, N1c = nc + 1;
@@ -1389,12 +1342,14 @@ cudaError_t coef(cudaStream_t s, const Grid& g, const T* kappa, T* coef, int64_t
 template <class T>
 cudaError_t pcg_pq(cudaStream_t s, const Grid& g, const T* kappa, const T* z, const T* p_old,
                    T* p_new, T* q, const Scalars& sc, double* part, int64_t B, Prof p, const T* coef) {
-  if (coef)
-    k_pq2<T, true><<<sgrid(g, B), SBLOCK, 0, s>>>(g, coef, coef_stride(g), z, p_old, p_new, q, sc.beta,
-                                                  sc.active, part, p);
-  else
-    k_pq2<T, false><<<sgrid(g, B), SBLOCK, 0, s>>>(g, kappa, g.es, z, p_old, p_new, q, sc.beta, sc.active,
-                                                   part, p);
+  if constexpr (sizeof(T) == 8) {   // the FP32 stencils run on kappa
+    if (coef) {
+      k_pq2<T, true><<<sgrid(g, B), SBLOCK, 0, s>>>(g, coef, coef_stride(g), z, p_old, p_new, q, sc.beta,
+                                                    sc.active, part, p);
+      return cudaGetLastError();
+    }
+  }
+  k_pq2<T, false><<<sgrid(g, B), SBLOCK, 0, s>>>(g, kappa, g.es, z, p_old, p_new, q, sc.beta, sc.active, part, p);
   return cudaGetLastError();
 }
 
@@ -1417,10 +1372,13 @@ cudaError_t mg_pre(cudaStream_t s, const Grid& g, const T* kappa, const T* w, co
                    T* r1, const int32_t* active, int64_t B, Prof p, const T* coef) {
   with_strips<T>(g, B, [&](auto sr, dim3 grid) {
     constexpr int SR = decltype(sr)::value;
-    if (coef)
-      k_mgpre2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coef, coef_stride(g), w, b, e, r1, active, p);
-    else
-      k_mgpre2<T, false, SR><<<grid, SBLOCK, 0, s>>>(g, kappa, g.es, w, b, e, r1, active, p);
+    if constexpr (sizeof(T) == 8) {
+      if (coef) {
+        k_mgpre2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coef, coef_stride(g), w, b, e, r1, active, p);
+        return;
+      }
+    }
+    k_mgpre2<T, false, SR><<<grid, SBLOCK, 0, s>>>(g, kappa, g.es, w, b, e, r1, active, p);
   });
   return cudaGetLastError();
 }
@@ -1461,14 +1419,12 @@ cudaError_t mg_post(cudaStream_t s, const Grid& g, const Grid& coarse, const T* 
                     double* part, int64_t B, Prof p, const T* coef) {
   const auto launch = [&](auto sr, dim3 grid) {
     constexpr int SR = decltype(sr)::value;
-    if (coef)
-      k_mgpost2<T, true, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, coef, coef_stride(g), w, b, e, ec, out,
-                                                        active, part, p);
-    else if constexpr (sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4)
       k_mgpost2f<SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, w, b, ec, out, active, part, p);
+    else if (coef)
+      k_mgpost2<true, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, coef, coef_stride(g), w, b, e, ec, out, active, part, p);
     else
-      k_mgpost2<T, false, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, g.es, w, b, e, ec, out,
-                                                         active, part, p);
+      k_mgpost2<false, SR><<<grid, SBLOCK, 0, s>>>(g, coarse.ns, kappa, g.es, w, b, e, ec, out, active, part, p);
   };
   if (part)
     launch(std::integral_constant<int, SROWS>{}, sgrid(g, B));
