@@ -37,10 +37,7 @@ namespace {
 constexpr int EXP_TAB = 64;
 __device__ double g_exp2_tab[EXP_TAB];
 constexpr double kInvLn2x64 = 92.332482616893658071;   // 64 / ln 2
-// ln 2 / 64 = 0.0108304246962491454596... as L1 (32 significant bits) + L2
-constexpr double kLn2d64Hi = 0x1.62e42fee00000p-7;     // 0.01083042469326755963265895843505859375
-constexpr double kLn2d64Lo = 2.9815858269852934627254151261796896e-12;
-constexpr double kR = kLn2d64Hi + kLn2d64Lo;
+constexpr double kR = 0x1.62e42fefa39efp-7;            // ln 2 / 64 = 0.0108304246962491454596...
 constexpr double kRound = 6755399441055744.0;          // 1.5 2^52
 constexpr int kBig = 0x40ef0000;                       // high word of |t| = 64 * 992 (|x| = 687.6)
 
