@@ -47,7 +47,7 @@ def parse():
                     help="profile case: 3D FP32 stencil tile shape (mlmc_config.stencil_tile)")
     ap.add_argument("--profile-kle", action="store_true",
                     help="profiling case: the KLE contraction of the finest level's batch "
-                         "(--profile-batch samples), FP64 and tensor-core kernels, twice each")
+                         "(--profile-batch samples), FP64 and FP32 kernels, twice each")
     ap.add_argument("--form", default="fp64", choices=["fp64", "mixed"],
                     help="form of the headline line (the other form is measured alongside)")
     ap.add_argument("--single-form", action="store_true")
@@ -687,10 +687,10 @@ def bench_ours(args):
     if os.path.exists(pk_path):
         peaks = json.load(open(pk_path))
     # the mixed form with its FP32 kappa made directly (kle_tensor = 1)
-    kle_tc = None
+    kle32 = None
     if not args.single_form and "mixed" in forms:
         cfg = m.config_from_workload(wl, precision="mixed", kle_tensor=1)
-        kle_tc = measure_form(m, wl, cfg, stream, args, world, barrier, with_e2e=False, rank=rank,
+        kle32 = measure_form(m, wl, cfg, stream, args, world, barrier, with_e2e=False, rank=rank,
                               gather=gather)
     main = forms[args.form]
     ms = reduce_max(main["ms"])
@@ -713,13 +713,13 @@ def bench_ours(args):
                        "autotune": res["tune"],
                        "roofline": roofline_of(res, peaks, fp64_alu=(form == "fp64"), dim=wl["dim"],
                                                fp64_probe=fp64_probe)}
-    if kle_tc is not None:
-        oms = reduce_max(kle_tc["ms"])
+    if kle32 is not None:
+        oms = reduce_max(kle32["ms"])
         other["mixed+kle_tensor"] = {
-            "value": kle_tc["dofs_step"] * args.steps / (oms / 1e3), "unit": "coupled DOF-solves/s",
-            "ms_per_step": oms / args.steps, "samples_per_level": kle_tc["N"],
-            "q_hat": kle_tc["q"], "stat_var": kle_tc["v"], "gpu_launches": int(kle_tc["launches"]),
-            "kappa_share": kle_tc["shares"].get("kappa"), "autotune": kle_tc["tune"]}
+            "value": kle32["dofs_step"] * args.steps / (oms / 1e3), "unit": "coupled DOF-solves/s",
+            "ms_per_step": oms / args.steps, "samples_per_level": kle32["N"],
+            "q_hat": kle32["q"], "stat_var": kle32["v"], "gpu_launches": int(kle32["launches"]),
+            "kappa_share": kle32["shares"].get("kappa"), "autotune": kle32["tune"]}
     if rank == 0:
         names = {"fp64": "plain FP64", "mixed": "mixed: FP32 inner PCG + FP64 refinement",
                  "mixed+kle_tensor": "mixed, FP32 kappa made from the KLE coefficients"}
