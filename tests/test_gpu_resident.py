@@ -1,10 +1,12 @@
 """Small-mesh solves as one resident launch (csrc/resident.cu) against the
-oracle, at the sizes where its layout changes: one CTA or a cluster of 2, 4
-or 8 per sample, bands with an odd last slab, levels split or on one CTA, the
-largest meshes it takes and the first ones it leaves to the separate kernels.
+oracle, at the sizes where its layout changes: one CTA or a cluster of 2, 4, 8
+or (Jacobi) 16 per sample, bands with an odd last slab, levels split or on one
+CTA, the largest meshes it takes and the first ones it leaves to the separate
+kernels (3D multigrid: 32^3, in test_gpu_parity3d.py).
 
 Tolerances: the solve stops at ||r|| <= 1e-11 ||b||, so Q is within 1e-9 and u
 within 1e-7 of the oracle's direct solution (the bounds of the other solves)."""
+import functools
 from fractions import Fraction
 
 import numpy as np
@@ -48,21 +50,27 @@ def solve(m, dim, n, solver, precision, kap, **over):
 
 
 SIZES = [(2, "gmg", n) for n in (2, 4, 8, 16, 32, 64, 128, 256)] + \
-        [(2, "jacobi", n) for n in (2, 3, 23, 33, 45, 100, 131, 235, 236)] + \
-        [(3, "gmg", n) for n in (4, 8, 16, 32)] + [(3, "jacobi", n) for n in (3, 9, 13, 18, 32, 33)]
+        [(2, "jacobi", n) for n in (2, 3, 23, 33, 45, 67, 100, 131, 170, 171, 256, 257)] + \
+        [(3, "gmg", n) for n in (4, 8, 16)] + [(3, "jacobi", n) for n in (3, 9, 13, 18, 24, 25, 30, 31)]
+
+
+@functools.lru_cache(maxsize=None)
+def reference(dim, n):
+    """Element coefficients and the oracle's solutions (the larger 3D meshes, slow there: one sample)."""
+    kap = random_element_field(dim, n, 2 if n ** dim < 20 ** 3 or dim == 2 else 1, seed=11 * n + dim, spread=0.7)
+    b = fem.load_vector(dim, n)
+    return kap, [fem.solve(fem.assemble_fast(dim, n, k), b, dim) for k in kap]
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("dim,solver,n", SIZES)
 def test_solve_matches_oracle(m, dim, solver, n, precision):
-    count = 2
-    kap = random_element_field(dim, n, count, seed=11 * n + dim, spread=0.7)
+    kap, refs = reference(dim, n)
     qoi = "box" if n % 4 == 0 else "domain"
     st, u, q, it = solve(m, dim, n, solver, precision, kap, qoi=qoi)
     assert st == 0 and np.all(it > 0)
-    b, w = fem.load_vector(dim, n), fem.qoi_weights(dim, n, qoi)
-    for s in range(count):
-        ref = fem.solve(fem.assemble_fast(dim, n, kap[s]), b, dim)
+    w = fem.qoi_weights(dim, n, qoi)
+    for s, ref in enumerate(refs):
         assert abs(q[s] - w @ ref) <= 1e-9 * abs(w @ ref)
         assert np.max(np.abs(fem.from_node_grid(dim, n, u[s]) - ref)) <= 1e-7 * np.max(np.abs(ref))
         # boundary nodes are written as 0
@@ -91,8 +99,10 @@ def test_the_meshes_that_run_resident(m, dim, solver, precision, last, first_lef
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
-@pytest.mark.parametrize("dim,solver,n", [(2, "gmg", 64), (2, "jacobi", 45), (3, "gmg", 16), (2, "gmg", 8)])
+@pytest.mark.parametrize("dim,solver,n", [(2, "gmg", 64), (2, "jacobi", 45), (3, "gmg", 16), (2, "gmg", 8),
+                                          (2, "jacobi", 67), (2, "jacobi", 100), (3, "jacobi", 18), (3, "jacobi", 23)])
 def test_results_do_not_depend_on_the_batch(m, dim, solver, n, precision):
+    """One band per CTA alone, two or four in the batch (Jacobi from 66^2 and 18^3 on: 16 bands)."""
     kap = random_element_field(dim, n, 200, seed=5, spread=0.5)
     _, u, q, it = solve(m, dim, n, solver, precision, kap)
     for s in (0, 7, 199):
@@ -154,7 +164,8 @@ def test_fused_levels_do_not_depend_on_the_batch(m, dim, n, precision, count):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
-@pytest.mark.parametrize("dim,solver,n0,count", [(2, "gmg", 32, 130), (2, "jacobi", 22, 150), (3, "gmg", 8, 150)])
+@pytest.mark.parametrize("dim,solver,n0,count", [(2, "gmg", 32, 130), (2, "jacobi", 22, 150), (3, "gmg", 8, 150),
+                                                 (2, "jacobi", 50, 64), (3, "jacobi", 9, 130)])
 def test_coupled_batches_repeat_bitwise(m, dim, solver, n0, count, precision):
     """CTAs of several bands: a batch gives the same bits every time, and each sample the bits of a call of its own."""
     wl = small_case(dim, n0=n0, levels=2, m=3, solver=solver, precision=precision)
